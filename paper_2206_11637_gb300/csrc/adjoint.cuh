@@ -45,34 +45,6 @@ constexpr int adj_minb() {
 // forward recomputation, doubled the adjoint's time on the same bubble: 831 ->
 // 1691 ms.  It is not used.)
 
-// The step's parameters in the arithmetic type R, converted once on the host:
-// converting the doubles of Phys in every thread kept the FP64 pipe (1/64 of
-// the FP32 rate on this part) three quarters busy in k_adj_local.  (The fused
-// forward step keeps Phys: the same change there measured 2.6 % slower in
-// FP16S and 0.9 % in FP32, its schedule losing more to load latency than the
-// conversions cost.)
-template <typename R>
-struct PhysR {
-  R rho_l, drho, tau_l, dtau, beta, kappa, inv_xi, omega_phi, gx, gy, gz;
-};
-
-template <typename R>
-inline PhysR<R> phys_r(const Phys& p) {
-  PhysR<R> q;
-  q.rho_l = (R)p.rho_l;
-  q.drho = (R)(p.rho_h - p.rho_l);
-  q.tau_l = (R)p.tau_l;
-  q.dtau = (R)(p.tau_h - p.tau_l);
-  q.beta = (R)p.beta;
-  q.kappa = (R)p.kappa;
-  q.inv_xi = (R)p.inv_xi;
-  q.omega_phi = (R)p.omega_phi;
-  q.gx = (R)p.gx;
-  q.gy = (R)p.gy;
-  q.gz = (R)p.gz;
-  return q;
-}
-
 // Parameters of the reverse sweep that the forward step folds into Phys.
 struct AdjPar {
   double M, xi, sigma;

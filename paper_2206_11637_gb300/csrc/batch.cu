@@ -47,6 +47,8 @@ pfl_status bfail(pfl_status s, const std::string& m) {
 struct BInst {
   Geo32 geo;
   Phys ph;
+  StepV<1>::Par ph32;  // ph in the arithmetic types of the FP32 and FP64 steps
+  StepV<0>::Par ph64;
   void* h[2];   // the two array pairs of the fused step
   void* g[2];
   void* phi;    // phi written by the steps (phi of the state each step started from)
@@ -78,13 +80,13 @@ constexpr int GRAPH_PAIRS = 8;  // a graph holds 2 * GRAPH_PAIRS lattice steps
 // zero at launch; the last block to finish zeroes them for the next launch,
 // which stream order puts after this one.
 template <int PREC, int TX, int TY, int FLAT>
-__global__ void __launch_bounds__(TX * TY, (PREC == 0 ? PFL_ZM_MINB_FP64 : PFL_ZM_MINB) * ZM_TX * ZM_TY / (TX * TY))
+__global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
     k_batch_zm(const BInst* __restrict__ inst, const BTile* __restrict__ tiles, int ntiles, int ab,
                unsigned* __restrict__ ctr) {
   typedef typename Store<PREC>::S S;
   typedef typename Store<PREC>::PhiT PhiT;
   __shared__ Geo32 sgeo;
-  __shared__ Phys sph;
+  __shared__ typename StepV<PREC>::Par sph;
   __shared__ int sact;
   __shared__ void* sptr[5];
   __shared__ int szc;
@@ -102,7 +104,10 @@ __global__ void __launch_bounds__(TX * TY, (PREC == 0 ? PFL_ZM_MINB_FP64 : PFL_Z
     if (tid == 0) {
       const BInst* I = inst + tile.inst;
       sgeo = I->geo;
-      sph = I->ph;
+      if constexpr (PREC == 0)
+        sph = I->ph64;
+      else
+        sph = I->ph32;
       sact = I->active;
       sptr[0] = I->h[ab];
       sptr[1] = I->g[ab];
@@ -591,6 +596,8 @@ pfl_status pfl_batch_init(const pfl_params* params, int count, const double* con
       return bfail(PFL_ERR_STATE, "integer divider self-check failed");
     }
     I.ph = phys_of(&q);
+    I.ph32 = step_par<1>(I.ph);
+    I.ph64 = step_par<0>(I.ph);
     char* at = b->ws + L.off[i];
     for (int pr = 0; pr < 2; ++pr) {
       I.h[pr] = at;

@@ -205,6 +205,7 @@ void launch_phi(pfl_ctx* c) {
 template <int PREC, int QH, int BGK>
 void step_only(pfl_ctx* c) {
   const unsigned nb = blocks_for(c->geo.N, 256);
+  const typename StepV<PREC>::Par ph1 = step_par<PREC>(c->ph);
   if (c->zm) {
     const int ty = zm_ty(c->p.nz == 1);
     const dim3 grid((c->p.nx + ZM_TX - 1) / ZM_TX, (c->p.ny + ty - 1) / ty, (c->p.nz + c->zc - 1) / c->zc);
@@ -225,7 +226,7 @@ void step_only(pfl_ctx* c) {
     const unsigned long long* tclock = c->capturing ? clock_of(c) : nullptr;
     const int tofs = (int)(c->t - c->cap_t0);
 #define PFL_ZM(FLAT, SOLID)                                                                                   \
-  cudaLaunchKernelEx(&cfg, k_step_zm<PREC, QH, FLAT, SOLID>, c->g32, c->ph, ha, ga, hnext<PREC>(c),           \
+  cudaLaunchKernelEx(&cfg, k_step_zm<PREC, QH, FLAT, SOLID>, c->g32, ph1, ha, ga, hnext<PREC>(c),            \
                      gnext<PREC>(c), shift, phicur<PREC>(c), c->zc, step_seed(c), links, tclock, tofs,       \
                      (const __half*)pgshift(c), pgcur(c))
     if (c->p.nz == 1) {
@@ -257,11 +258,11 @@ void step_only(pfl_ctx* c) {
   } else {
     const unsigned nbm = blocks_for(c->geo.N, PFL_STEP_THREADS);
     if (c->swapped)
-      k_step_mrt<PREC, QH, 1><<<nbm, PFL_STEP_THREADS, 0, c->stream>>>(c->g32, c->ph, hbuf<PREC>(c), gbuf<PREC>(c),
+      k_step_mrt<PREC, QH, 1><<<nbm, PFL_STEP_THREADS, 0, c->stream>>>(c->g32, ph1, hbuf<PREC>(c), gbuf<PREC>(c),
                                                                     phicur<PREC>(c), phishift<PREC>(c), step_seed(c),
                                                                     pgshift(c), pgcur(c));
     else
-      k_step_mrt<PREC, QH, 0><<<nbm, PFL_STEP_THREADS, 0, c->stream>>>(c->g32, c->ph, hbuf<PREC>(c), gbuf<PREC>(c),
+      k_step_mrt<PREC, QH, 0><<<nbm, PFL_STEP_THREADS, 0, c->stream>>>(c->g32, ph1, hbuf<PREC>(c), gbuf<PREC>(c),
                                                                     phicur<PREC>(c), phishift<PREC>(c), step_seed(c),
                                                                     pgshift(c), pgcur(c));
   }
@@ -1238,10 +1239,11 @@ void zm_step_slots(pfl_ctx* c, const SlotPtr<PREC>& a, const SlotPtr<PREC>& b) {
   const int ty = zm_ty(c->p.nz == 1);
   const dim3 grid((c->p.nx + ZM_TX - 1) / ZM_TX, (c->p.ny + ty - 1) / ty, (c->p.nz + c->zc - 1) / c->zc);
   const dim3 block(ZM_TX, ty);
+  const typename StepV<PREC>::Par ph = step_par<PREC>(c->ph);
   if (c->p.nz == 1)
-    k_step_zm<PREC, QH, 1><<<grid, block, 0, c->stream>>>(c->g32, c->ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc, 0u);
+    k_step_zm<PREC, QH, 1><<<grid, block, 0, c->stream>>>(c->g32, ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc, 0u);
   else
-    k_step_zm<PREC, QH, 0><<<grid, block, 0, c->stream>>>(c->g32, c->ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc, 0u);
+    k_step_zm<PREC, QH, 0><<<grid, block, 0, c->stream>>>(c->g32, ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc, 0u);
 }
 
 // Adjoint with the fused two-array engine.  Forward sweep: checkpoints every K

@@ -7,8 +7,7 @@
 // quadratic polynomial of its velocity,
 //   f+_i / w_i = alpha + beta . c_i + c_i . Gamma . c_i,
 // so a pair (c, -c) shares E = alpha + c.Gamma.c and differs only in the sign
-// of L = beta . c.  Moments are gathered the same way: S = f_c + f_-c feeds the
-// even moments (p*, phi, second moments), D = f_c - f_-c the odd ones.
+// of L = beta . c.
 //   g:  alpha = p* - 3/2 u.u - a2 tr(Pi^d)/3,  beta = 3 u + 3/2 F / rho,
 //       Gamma = 9/2 u u^T + a2 Pi^d,           a2 = 9/2 (1 - omega)
 //   h:  alpha = phi - a2 tr(Pi^dh)/3,           beta = 3 phi u + a1 J^d + (1 - omega_phi/2) theta n,
@@ -22,9 +21,9 @@
 // crosses a no-slip face; offsets of a direction are sums of these, fixed at
 // compile time inside the unrolled loops.
 #pragma once
-#include <type_traits>
 
 #include "kernels.cuh"
+#include "vec.cuh"
 
 #ifndef PFL_STEP_THREADS
 #define PFL_STEP_THREADS 128
@@ -32,10 +31,10 @@
 #ifndef PFL_STEP_MINB
 #define PFL_STEP_MINB 4
 #endif
-// Resident blocks per SM the fused step is compiled for.  Three (80 registers,
-// a few bytes of spill) beat two (128 registers) by 13-20 % for FP16S: the
-// kernel is latency-bound and gains from the extra warps.  FP64, bound by the
-// FP64 units, keeps two (three would spill ~200 bytes per thread).
+// Resident blocks of 256 threads per SM the fused step is compiled for.  Three
+// (80 registers) against two (128) and four (64, with spills) on a 256x192x256
+// impact: FP16S 15.7, 14.5 and 14.5 GLUPS; FP32 14.4, 14.4 and 6.2 (its L1
+// prefetch then overflows).  FP64, bound by the FP64 units, keeps two.
 #ifndef PFL_ZM_MINB
 #define PFL_ZM_MINB 3
 #endif
@@ -46,7 +45,8 @@
 // next, issued one plane ahead right after the plane barrier (1; 0 = none).
 // Measured on the 128x384x128 bubble: FP32 14.0 -> 14.9 GLUPS.  FP16S (issue
 // bound) lost 5 %, single-plane lattices 8-10 % and the D3Q27 phase field 1 %
-// (10.94 -> 10.82), so they take none.
+// (10.94 -> 10.82), so they take none.  (The h populations of the plane filled
+// next as well: 15.0 -> 12.5 GLUPS on a 256x192x256 impact.)
 #ifndef PFL_ZM_PREFETCH
 #define PFL_ZM_PREFETCH 1
 #endif
@@ -61,16 +61,6 @@
 #ifndef PFL_ZM_PDL
 #define PFL_ZM_PDL 1
 #endif
-// Interior form of the fused step (1; 0 = the general form everywhere): blocks
-// clear of the lattice's faces by two cells take neighbour offsets without
-// wall, wrap or solid tests.  Measured on the 512x384x512 impact (events, 128
-// steps): FP16S 13.5 GLUPS with it against 16.1 without, FP32 14.5 against
-// 14.8 -- the second copy of the unrolled body costs more than the tests it
-// saves -- so it is off.
-#ifndef PFL_ZM_INTERIOR
-#define PFL_ZM_INTERIOR 0
-#endif
-
 namespace pfl {
 
 // Exact q = n / d for 32-bit unsigned n and a divisor fixed for the launch
@@ -186,18 +176,6 @@ struct CellOff {
   }
 };
 
-// Offsets of a cell whose neighbours two cells deep all lie inside the lattice
-// (no face, no wrap, no solid): every link is valid and the offset of
-// direction c is cx + cy sy + cz sz.  The fused step takes this form for blocks
-// whose tile, ring and z range stay clear of the lattice's faces.
-struct CellOffI {
-  int sy, sz;
-  static constexpr unsigned blk = 0;
-  __device__ __forceinline__ int off(int cx, int cy, int cz) const { return cx + cy * sy + cz * sz; }
-  __device__ __forceinline__ constexpr bool valid(int, int, int) const { return true; }
-  __device__ __forceinline__ int soff(int cx, int cy, int cz) const { return off(cx, cy, cz); }
-};
-
 // Raw stored value as the arithmetic type (FP16: the stored number, unscaled).
 template <int PREC>
 __device__ __forceinline__ typename Store<PREC>::R raw(typename Store<PREC>::S v) {
@@ -270,21 +248,6 @@ __device__ __forceinline__ typename Store<PREC>::S pack_sr(typename Store<PREC>:
   }
 }
 
-// w (s + r) for a lattice weight w, s the large part of a stored population
-// (phi or p*) and r the small rest.  FP32 carries w as hi + lo: the FP32
-// roundings of the D3Q15 weights alone sum to 1 + 7.5e-9 (D3Q27 likewise),
-// a bias of the zeroth and second moments that repeats every step and, over
-// 1000 steps, was the largest FP32 error of phi and u.  FP64 uses w as is.
-template <typename R>
-__device__ __forceinline__ R wsum(double w, R s, R r) {
-  if constexpr (sizeof(R) == 4) {
-    const float hi = (float)w, lo = (float)(w - (double)hi);
-    return fmaf(hi, s, fmaf(lo, s, hi * r));
-  } else {
-    return fma(w, s, w * r);
-  }
-}
-
 __device__ __forceinline__ void cell_off(const Geo32& geo, unsigned c, CellOff& o) {
   const unsigned yz = fdiv(c, geo.dx);
   const unsigned x = c - yz * geo.nx;
@@ -316,10 +279,637 @@ __device__ __forceinline__ void load_pair(const typename Store<PREC>::S* __restr
   }
 }
 
+
+// ---------------------------------------------------------------------------
+// Moments.  A population set is a tensor product (D3Q27, D2Q9) or its axis and
+// corner part (D3Q15), so the moments up to second order fall out of sums and
+// differences along x, then y, then z: 66 operations for the ten moments of
+// D3Q27 against 111 by opposite pairs, 39 against 63 for D3Q15.
+// ld(cx, cy, cz) gives the population of direction c.  W = 0: populations as
+// they are; W = 1: values divided by their lattice weight, summed with the
+// weights times 216 (D3Q27: (1, 4, 1) per axis), 36 (D2Q9) or 72 (D3Q15: corners
+// 1, axes 8, rest 16), exact multiples.
+template <class V>
+struct Mom {
+  V s, x, y, z, xx, yy, zz, xy, yz, xz;  // sum f, sum c f, sum c c f
+};
+template <int Q>
+__host__ __device__ constexpr double wsum_of() {
+  return Q == 27 ? 216.0 : (Q == 9 ? 36.0 : 72.0);
+}
+// index of direction c in the lattice's order
+template <int Q>
+__host__ __device__ constexpr int lq_index(int cx, int cy, int cz) {
+  const int i = 9 * (cz + 1) + 3 * (cy + 1) + cx + 1;
+  return Q == 27 ? i : (Q == 9 ? i - 9 : (i < 13 ? i / 2 : (i == 13 ? 7 : i / 2 + 1)));
+}
+
+template <int W, class V>
+__device__ __forceinline__ V sum3(V a, V b, V c) {  // a + b + c, or a + 4 b + c
+  if constexpr (W)
+    return vfma(vbc<V>(4.0), b, a + c);
+  else
+    return (a + c) + b;
+}
+
+template <class V>
+struct PlaneMom {
+  V m00, m10, m20, m01, m11, m02;  // x-order, y-order within one z plane
+};
+template <int W, class V, class LD>
+__device__ __forceinline__ PlaneMom<V> plane_mom(const LD& ld, int cz) {
+  V a0[3], a1[3], a2[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const V l = ld(-1, j - 1, cz), c = ld(0, j - 1, cz), r = ld(1, j - 1, cz);
+    a0[j] = sum3<W>(l, c, r);
+    a1[j] = r - l;
+    a2[j] = l + r;
+  }
+  PlaneMom<V> p;
+  p.m00 = sum3<W>(a0[0], a0[1], a0[2]);
+  p.m01 = a0[2] - a0[0];
+  p.m02 = a0[0] + a0[2];
+  p.m10 = sum3<W>(a1[0], a1[1], a1[2]);
+  p.m11 = a1[2] - a1[0];
+  p.m20 = sum3<W>(a2[0], a2[1], a2[2]);
+  return p;
+}
+
+template <int Q, int W, class V, class LD>
+__device__ __forceinline__ Mom<V> moments(const LD& ld) {
+  Mom<V> m;
+  if constexpr (Q == 27) {
+    const PlaneMom<V> a = plane_mom<W, V>(ld, -1), b = plane_mom<W, V>(ld, 0), c = plane_mom<W, V>(ld, 1);
+    m.s = sum3<W>(a.m00, b.m00, c.m00);
+    m.z = c.m00 - a.m00;
+    m.zz = a.m00 + c.m00;
+    m.x = sum3<W>(a.m10, b.m10, c.m10);
+    m.xz = c.m10 - a.m10;
+    m.y = sum3<W>(a.m01, b.m01, c.m01);
+    m.yz = c.m01 - a.m01;
+    m.xx = sum3<W>(a.m20, b.m20, c.m20);
+    m.yy = sum3<W>(a.m02, b.m02, c.m02);
+    m.xy = sum3<W>(a.m11, b.m11, c.m11);
+  } else if constexpr (Q == 9) {
+    const PlaneMom<V> b = plane_mom<W, V>(ld, 0);
+    m.s = b.m00;
+    m.x = b.m10;
+    m.y = b.m01;
+    m.xx = b.m20;
+    m.yy = b.m02;
+    m.xy = b.m11;
+    m.z = m.zz = m.yz = m.xz = vbc<V>(0.0);
+  } else {
+    PlaneMom<V> p[2];  // corners of the planes cz = -1, 1: m00, m10, m01, m11
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const V a = ld(-1, -1, 2 * k - 1), b = ld(1, -1, 2 * k - 1), c = ld(-1, 1, 2 * k - 1), d = ld(1, 1, 2 * k - 1);
+      const V r0 = a + b, r1 = c + d, e0 = b - a, e1 = d - c;
+      p[k].m00 = r0 + r1;
+      p[k].m01 = r1 - r0;
+      p[k].m10 = e0 + e1;
+      p[k].m11 = e1 - e0;
+    }
+    const V c0 = p[0].m00 + p[1].m00;
+    const V xm = ld(-1, 0, 0), xp = ld(1, 0, 0), ym = ld(0, -1, 0), yp = ld(0, 1, 0), zm = ld(0, 0, -1),
+            zp = ld(0, 0, 1), r = ld(0, 0, 0);
+    const V sx = xm + xp, sy = ym + yp, sz = zm + zp, dx = xp - xm, dy = yp - ym, dz = zp - zm;
+    const V cx = p[0].m10 + p[1].m10, cy = p[0].m01 + p[1].m01, cz = p[1].m00 - p[0].m00;
+    if constexpr (W) {
+      const V w8 = vbc<V>(8.0);
+      m.s = vfma(vbc<V>(16.0), r, vfma(w8, (sx + sy) + sz, c0));
+      m.x = vfma(w8, dx, cx);
+      m.y = vfma(w8, dy, cy);
+      m.z = vfma(w8, dz, cz);
+      m.xx = vfma(w8, sx, c0);
+      m.yy = vfma(w8, sy, c0);
+      m.zz = vfma(w8, sz, c0);
+    } else {
+      m.s = (c0 + ((sx + sy) + sz)) + r;
+      m.x = cx + dx;
+      m.y = cy + dy;
+      m.z = cz + dz;
+      m.xx = c0 + sx;
+      m.yy = c0 + sy;
+      m.zz = c0 + sz;
+    }
+    m.xy = p[0].m11 + p[1].m11;
+    m.xz = p[1].m10 - p[0].m10;
+    m.yz = p[1].m01 - p[0].m01;
+  }
+  return m;
+}
+
+// Moments of an FP16S set: f_i = w_i (s_i / K + shift of its writer), the
+// stored and the shift part summed apart (differences of large shifts cancel
+// exactly) and joined once.
+template <int Q, class V, class LD, class SH>
+__device__ __forceinline__ Mom<V> moments_f16(const LD& ld, const SH& sh, double K) {
+  const Mom<V> a = moments<Q, 1, V>(ld), b = moments<Q, 1, V>(sh);
+  const V k = vbc<V>(1.0 / K), n = vbc<V>(1.0 / wsum_of<Q>());
+  Mom<V> m;
+  m.s = vfma(k, a.s, b.s) * n;
+  m.x = vfma(k, a.x, b.x) * n;
+  m.y = vfma(k, a.y, b.y) * n;
+  m.z = vfma(k, a.z, b.z) * n;
+  m.xx = vfma(k, a.xx, b.xx) * n;
+  m.yy = vfma(k, a.yy, b.yy) * n;
+  m.zz = vfma(k, a.zz, b.zz) * n;
+  m.xy = vfma(k, a.xy, b.xy) * n;
+  m.yz = vfma(k, a.yz, b.yz) * n;
+  m.xz = vfma(k, a.xz, b.xz) * n;
+  return m;
+}
+
+// FP32 moments by opposite pairs, in the order of the set's members: S = f_c +
+// f_-c feeds the even moments, D = f_c - f_-c the odd ones (see collide_pairs).
+template <int Q, class LD>
+__device__ __forceinline__ Mom<F1> moments_pairs(const LD& ld) {
+  float s = ld(0, 0, 0).v, x = 0, y = 0, z = 0, xx = 0, yy = 0, zz = 0, xy = 0, yz = 0, xz = 0;
+#pragma unroll
+  for (int i = 0; i < (Q - 1) / 2; ++i) {
+    const int cx = q27_cx(lq_to27<Q>(i)), cy = q27_cy(lq_to27<Q>(i)), cz = q27_cz(lq_to27<Q>(i));
+    const float a = ld(cx, cy, cz).v, b = ld(-cx, -cy, -cz).v;
+    const float S = a + b, D = a - b;
+    s += S;
+    if (cx) x += cx > 0 ? D : -D;
+    if (cy) y += cy > 0 ? D : -D;
+    if (cz) z += cz > 0 ? D : -D;
+    if (cx) xx += S;
+    if (cy) yy += S;
+    if (cz) zz += S;
+    if (cx && cy) xy += (cx * cy > 0) ? S : -S;
+    if (cy && cz) yz += (cy * cz > 0) ? S : -S;
+    if (cx && cz) xz += (cx * cz > 0) ? S : -S;
+  }
+  return Mom<F1>{F1{s}, F1{x}, F1{y}, F1{z}, F1{xx}, F1{yy}, F1{zz}, F1{xy}, F1{yz}, F1{xz}};
+}
+
+// The h moments of a cell (ld: raw stored values, sh: the phi shift of each
+// population's writer, read for FP16S only); m.s is phi.  Everything that
+// forms phi goes through here (a caller that uses m.s alone leaves the rest to
+// dead-code elimination), so all phi of a state agree bitwise.
+template <int PREC, int QH, class V, class LD, class SH>
+__device__ __forceinline__ Mom<V> h_moments(const LD& ld, const SH& sh) {
+  if constexpr (PREC == 2)
+    return moments_f16<QH, V>(ld, sh, KH16);
+  else if constexpr (PREC == 1)
+    return moments_pairs<QH>(ld);
+  else
+    return moments<QH, 0, V>(ld);
+}
+template <int PREC, int QG, class V, class LD, class SH>
+__device__ __forceinline__ Mom<V> g_moments(const LD& ld, const SH& sh) {
+  if constexpr (PREC == 2)
+    return moments_f16<QG, V>(ld, sh, KG16);
+  else if constexpr (PREC == 1)
+    return moments_pairs<QG>(ld);
+  else
+    return moments<QG, 0, V>(ld);
+}
+
+// ---------------------------------------------------------------------------
+// The phi stencil.  The weights factor per axis, w1 = (1/6, 2/3, 1/6) =
+// 1 + delta^2 / 6 with delta^2 f = (f(-1) - f) + (f(+1) - f), so
+//   grad_x = 1/2 (1 + delta_y^2 / 6)(1 + delta_z^2 / 6)(phi(x+1) - phi(x-1)),
+//   lap    = 6 [(1 + delta_x^2 / 6)(1 + delta_y^2 / 6)(1 + delta_z^2 / 6) - 1] phi
+//          = q + delta_z^2 phi + delta_z^2 q / 6,  q = dx + delta_y^2 phi + delta_y^2 dx / 6,
+//            dx = delta_x^2 phi,
+// all in differences that are exact for nearby values.  The in-plane part (28
+// operations on nine values) is formed once per plane and kept while the march
+// passes; joining three planes takes 22 more: 50 per cell and nine reads
+// against about 130 and 27 by opposite pairs.  On one z plane (its own
+// neighbour) the z part vanishes exactly.
+template <class V>
+struct PhiPlane {
+  V c, q, gx, gy;
+};
+template <class V, class AT>
+__device__ __forceinline__ PhiPlane<V> phi_plane(const AT& at) {  // at(cx, cy)
+  const V w6 = vbc<V>(1.0 / 6.0);
+  V c[3], d[3], g[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const V l = at(-1, j - 1), r = at(1, j - 1);
+    c[j] = at(0, j - 1);
+    d[j] = (l - c[j]) + (r - c[j]);
+    g[j] = r - l;
+  }
+  PhiPlane<V> p;
+  p.c = c[1];
+  p.gx = vfma(w6, (g[0] - g[1]) + (g[2] - g[1]), g[1]);
+  p.gy = vfma(w6, d[2] - d[0], c[2] - c[0]);
+  p.q = vfma(w6, (d[0] - d[1]) + (d[2] - d[1]), d[1] + ((c[0] - c[1]) + (c[2] - c[1])));
+  return p;
+}
+template <class V>
+struct Grad {
+  V x, y, z, lap;
+};
+template <class V>
+__device__ __forceinline__ Grad<V> phi_grad(const PhiPlane<V>& m, const PhiPlane<V>& o, const PhiPlane<V>& p) {
+  const V w6 = vbc<V>(1.0 / 6.0), half = vbc<V>(0.5);
+  Grad<V> r;
+  r.x = half * vfma(w6, (m.gx - o.gx) + (p.gx - o.gx), o.gx);
+  r.y = half * vfma(w6, (m.gy - o.gy) + (p.gy - o.gy), o.gy);
+  r.z = half * vfma(w6, p.q - m.q, p.c - m.c);
+  r.lap = o.q + vfma(w6, (m.q - o.q) + (p.q - o.q), (m.c - o.c) + (p.c - o.c));
+  return r;
+}
+template <class V>
+__device__ __forceinline__ Grad<V> phi_grad_flat(const PhiPlane<V>& o) {  // phi_grad(o, o, o)
+  const V half = vbc<V>(0.5);
+  return Grad<V>{half * o.gx, half * o.gy, vbc<V>(0.0), o.q};
+}
+
+// ---------------------------------------------------------------------------
+// The step's parameters in the arithmetic type, formed once on the host.
+template <class V>
+struct PhysV {
+  V rho_l, drho, tau_l, dtau, beta4, mkappa, mdrho3, gx, gy, gz;
+  V c4;          // 4 (1 - omega_phi / 2) / xi
+  V a1;          // 3 (1 - omega_phi)
+  V a2, a2_3;    // 9 (1 - omega_phi), 3/2 (1 - omega_phi): 2 a2 and a2 / 3 of the h collision
+};
+template <class V>
+inline PhysV<V> phys_v(const Phys& p) {
+  PhysV<V> q;
+  q.rho_l = vbc<V>(p.rho_l);
+  q.drho = vbc<V>(p.rho_h - p.rho_l);
+  q.tau_l = vbc<V>(p.tau_l);
+  q.dtau = vbc<V>(p.tau_h - p.tau_l);
+  q.beta4 = vbc<V>(4.0 * p.beta);
+  q.mkappa = vbc<V>(-p.kappa);
+  q.mdrho3 = vbc<V>(-(p.rho_h - p.rho_l) / 3.0);
+  q.gx = vbc<V>(p.gx);
+  q.gy = vbc<V>(p.gy);
+  q.gz = vbc<V>(p.gz);
+  q.c4 = vbc<V>(4.0 * (1.0 - 0.5 * p.omega_phi) * p.inv_xi);
+  q.a1 = vbc<V>(3.0 * (1.0 - p.omega_phi));
+  q.a2 = vbc<V>(9.0 * (1.0 - p.omega_phi));
+  q.a2_3 = vbc<V>(1.5 * (1.0 - p.omega_phi));
+  return q;
+}
+
+// The same without the combined factors, in the arithmetic type R (the FP32
+// step and the adjoint).
+template <typename R>
+struct PhysR {
+  R rho_l, drho, tau_l, dtau, beta, kappa, inv_xi, omega_phi, gx, gy, gz;
+};
+
+template <typename R>
+inline PhysR<R> phys_r(const Phys& p) {
+  PhysR<R> q;
+  q.rho_l = (R)p.rho_l;
+  q.drho = (R)(p.rho_h - p.rho_l);
+  q.tau_l = (R)p.tau_l;
+  q.dtau = (R)(p.tau_h - p.tau_l);
+  q.beta = (R)p.beta;
+  q.kappa = (R)p.kappa;
+  q.inv_xi = (R)p.inv_xi;
+  q.omega_phi = (R)p.omega_phi;
+  q.gx = (R)p.gx;
+  q.gy = (R)p.gy;
+  q.gz = (R)p.gz;
+  return q;
+}
+
+// Arithmetic type of a cell, and the parameters its collision takes.
+template <int PREC>
+struct StepV {
+  typedef F1 T;
+  typedef PhysV<F1> Par;
+};
+template <>
+struct StepV<0> {
+  typedef D1 T;
+  typedef PhysV<D1> Par;
+};
+template <>
+struct StepV<1> {
+  typedef F1 T;
+  typedef PhysR<float> Par;
+};
+template <int PREC>
+inline typename StepV<PREC>::Par step_par(const Phys& p) {
+  if constexpr (PREC == 1)
+    return phys_r<float>(p);
+  else
+    return phys_v<typename StepV<PREC>::T>(p);
+}
+
+// Emits the post-collision pairs of a quadratic polynomial of the velocity,
+//   E = al + c . G . c (off-diagonal G doubled), L = b . c,
+// sharing the partial sums between directions: 21 additions for the even parts
+// and 10 for the odd ones of D3Q27 instead of 45 and 27.  put(i, oi, cx, cy,
+// cz, A, B): A for direction c (member i), B for -c (member oi).
+// F16: A = E + L, B = E - L (values divided by the weight).  Else the stored
+// value w (s + E +- L) with s the large part added last, one rounding at its
+// size.
+template <int Q, bool F16, class V, class PUT>
+__device__ __forceinline__ void emit_pairs(V s, V al, V bx, V by, V bz, V Gxx, V Gyy, V Gzz, V Gxy, V Gyz, V Gxz,
+                                           const PUT& put) {
+  const V Ex = al + Gxx, Ey = al + Gyy, Ez = al + Gzz;
+  const V Exy = Ex + Gyy, Exz = Ex + Gzz, Eyz = Ey + Gzz, E3 = Exy + Gzz;
+  const V p = E3 + Gxy, m = E3 - Gxy, sg = Gyz + Gxz, dg = Gyz - Gxz;
+  const V bxy = bx + by, bxny = bx - by;
+#pragma unroll
+  for (int i = 0; i < (Q - 1) / 2; ++i) {
+    const int cx = q27_cx(lq_to27<Q>(i)), cy = q27_cy(lq_to27<Q>(i)), cz = q27_cz(lq_to27<Q>(i));
+    const int n2 = cx * cx + cy * cy + cz * cz;
+    // (qx, qy, qz) = +-c with its first non-zero component positive
+    const int sgn = cx ? cx : (cy ? cy : cz);
+    const int qy = sgn * cy, qz = sgn * cz;
+    V E, L;
+    if (n2 == 1) {
+      E = cx ? Ex : (cy ? Ey : Ez);
+      L = cx ? bx : (cy ? by : bz);
+    } else if (n2 == 2) {
+      if (cx && cy) {
+        E = qy > 0 ? Exy + Gxy : Exy - Gxy;
+        L = qy > 0 ? bxy : bxny;
+      } else if (cx) {
+        E = qz > 0 ? Exz + Gxz : Exz - Gxz;
+        L = qz > 0 ? bx + bz : bx - bz;
+      } else {
+        E = qz > 0 ? Eyz + Gyz : Eyz - Gyz;
+        L = qz > 0 ? by + bz : by - bz;
+      }
+    } else {
+      E = qy > 0 ? (qz > 0 ? p + sg : p - sg) : (qz > 0 ? m - dg : m + dg);
+      const V b2 = qy > 0 ? bxy : bxny;
+      L = qz > 0 ? b2 + bz : b2 - bz;
+    }
+    V A, B;  // of +q and -q
+    if constexpr (F16) {
+      A = E + L;
+      B = E - L;
+    } else {
+      const double w = lq_w<Q>(i);
+      const V e = vbc<V>(w) * E;
+      A = vfma(vbc<V>(w), s, vfma(vbc<V>(w), L, e));
+      B = vfma(vbc<V>(w), s, vfma(vbc<V>(-w), L, e));
+    }
+    if (sgn > 0)
+      put(i, Q - 1 - i, cx, cy, cz, A, B);
+    else
+      put(i, Q - 1 - i, cx, cy, cz, B, A);
+  }
+}
+// the rest population of the same polynomial
+template <int Q, bool F16, class V>
+__device__ __forceinline__ V emit_rest(V s, V al) {
+  if constexpr (F16) return al;
+  const double w = lq_w<Q>((Q - 1) / 2);
+  return vfma(vbc<V>(w), s, vbc<V>(w) * al);
+}
+
+// The collision of both sets (moments to post-collision populations) of FP64
+// and FP16S, shared by every stream-collide kernel.
+//   pc, gr: phi^t of the cell and its stencil; gm: the g moments;
+//   hmom(): the h moments, read when their turn comes;
+//   out.shift(pst): FP16S, stores P = fp16(p*) of the cell and returns it;
+//   out.grest(v), out.g_(i, oi, cx, cy, cz, A, B), out.hrest(v), out.h_(...).
+template <int PREC, int QH, class V, class HM, class OUT>
+__device__ __forceinline__ void collide(const PhysV<V>& ph, V pc, const Grad<V>& gr, const Mom<V>& gm, const HM& hmom,
+                                        OUT& out) {
+  constexpr bool F16 = PREC == 2;
+  constexpr int QG = qg_of<QH>();  // D2Q9 with the 2-D phase field, else D3Q27
+  const V third = vbc<V>(1.0 / 3.0), one = vbc<V>(1.0), half = vbc<V>(0.5);
+  const V pst = gm.s;
+  V ux, uy, uz;
+  {
+    // ---- forces and velocity
+    const V rho = vfma(pc, ph.drho, ph.rho_l);
+    const V tau = vfma(pc, ph.dtau, ph.tau_l);
+    const V omega = vrcp(tau), rinv = vrcp(rho);
+    const V hr = half * rinv;
+    const V mu = vfma(ph.mkappa, gr.lap, ((ph.beta4 * pc) * (pc - one)) * (pc - half));
+    const V mc = vfma(pst, ph.mdrho3, mu);
+    V Fx = vfma(mc, gr.x, rho * ph.gx), Fy = vfma(mc, gr.y, rho * ph.gy), Fz = vfma(mc, gr.z, rho * ph.gz);
+    const V p3 = pst * third;
+    {
+      const V ax = vfma(Fx, hr, gm.x), ay = vfma(Fy, hr, gm.y), az = vfma(Fz, hr, gm.z);
+      const V nx = -ax, ny = -ay, nz = -az;
+      const V nxx = vfma(nx, ax, gm.xx - p3), nyy = vfma(ny, ay, gm.yy - p3), nzz = vfma(nz, az, gm.zz - p3);
+      const V nxy = vfma(nx, ay, gm.xy), nyz = vfma(ny, az, gm.yz), nxz = vfma(nx, az, gm.xz);
+      // -3 nu omega drho = -(1 - omega / 2) drho, since 3 nu = tau - 1/2
+      const V cm = vfma(half, omega, -one) * ph.drho;
+      Fx = vfma(cm, vfma(nxz, gr.z, vfma(nxy, gr.y, nxx * gr.x)), Fx);
+      Fy = vfma(cm, vfma(nyz, gr.z, vfma(nyy, gr.y, nxy * gr.x)), Fy);
+      Fz = vfma(cm, vfma(nzz, gr.z, vfma(nyz, gr.y, nxz * gr.x)), Fz);
+    }
+    ux = vfma(Fx, hr, gm.x);
+    uy = vfma(Fy, hr, gm.y);
+    uz = vfma(Fz, hr, gm.z);
+
+    // ---- g post-collision coefficients and pair stores.  FP16S scales them
+    // by the format's power of two and stores deviations from P = fp16(p*).
+    constexpr double K = F16 ? KG16 : 1.0;
+    const V mx = -ux, my = -uy, mz = -uz;
+    const V qx = mx * ux, qy = my * uy, qz = mz * uz;  // -u_a^2
+    // deviatoric second moments, (3 P_aa - p*) / 3 with one rounding: p* (1/3)
+    // would carry the rounded constant 1/3, a bias of 3e-8 p* that repeats
+    // every step
+    const V mp = -pst, three = vbc<V>(3.0);
+    const V dxx = vfma(vfma(three, gm.xx, mp), third, qx), dyy = vfma(vfma(three, gm.yy, mp), third, qy);
+    const V dzz = QG == 9 ? vbc<V>(0.0) : vfma(vfma(three, gm.zz, mp), third, qz);  // 2-D: the trace runs over x and y
+    const V a2 = vfma(vbc<V>(-4.5 * K), omega, vbc<V>(4.5 * K));
+    const V al = vfma(vbc<V>(1.5 * K), (qx + qy) + qz, (a2 * vbc<V>(-1.0 / 3.0)) * ((dxx + dyy) + dzz));
+    const V fr = vbc<V>(1.5 * K) * rinv, k3 = vbc<V>(3.0 * K);
+    const V bx = vfma(fr, Fx, k3 * ux), by = vfma(fr, Fy, k3 * uy), bz = vfma(fr, Fz, k3 * uz);
+    const V k45 = vbc<V>(-4.5 * K), k9 = vbc<V>(-9.0 * K), a22 = a2 + a2;
+    const V Gxx = vfma(k45, qx, a2 * dxx), Gyy = vfma(k45, qy, a2 * dyy), Gzz = vfma(k45, qz, a2 * dzz);
+    const V qxy = mx * uy, qyz = my * uz, qxz = mx * uz;
+    const V Gxy = vfma(k9, qxy, a22 * (gm.xy + qxy)), Gyz = vfma(k9, qyz, a22 * (gm.yz + qyz)),
+            Gxz = vfma(k9, qxz, a22 * (gm.xz + qxz));
+    V e0 = al;
+    if constexpr (F16) e0 = vfma(vbc<V>(K), pst - out.shift(pst), al);
+    out.grest(emit_rest<QG, F16>(pst, e0));
+    emit_pairs<QG, F16>(pst, e0, bx, by, bz, Gxx, Gyy, Gzz, Gxy, Gyz, Gxz,
+                        [&](int i, int oi, int cx, int cy, int cz, V A, V B) { out.g_(i, oi, cx, cy, cz, A, B); });
+  }
+
+  // ---- h post-collision coefficients and pair stores
+  {
+    constexpr double K = F16 ? KH16 : 1.0;
+    const Mom<V> h = hmom();
+    const V gn = vsqrt(vfma(gr.z, gr.z, vfma(gr.y, gr.y, gr.x * gr.x)));
+    // (1 - omega_phi / 2) theta / |grad phi|, theta = 4 phi (1 - phi) / xi
+    const V tn = vdiv((ph.c4 * pc) * (one - pc), gn + vbc<V>(1e-6));
+    // deviatoric second moments as (3 H_aa - phi) / 3 and the non-equilibrium
+    // flux J - phi u, one rounding each
+    const V mphi = -h.s, three = vbc<V>(3.0), a2_3 = F16 ? vbc<V>(K) * ph.a2_3 : ph.a2_3;
+    const V Gxx = a2_3 * vfma(three, h.xx, mphi), Gyy = a2_3 * vfma(three, h.yy, mphi);
+    const V Gzz = QG == 9 ? vbc<V>(0.0) : a2_3 * vfma(three, h.zz, mphi);
+    const V al = vbc<V>(-1.0 / 3.0) * ((Gxx + Gyy) + Gzz);
+    const V p3 = three * h.s;
+    V bx = vfma(p3, ux, vfma(ph.a1, vfma(mphi, ux, h.x), tn * gr.x));
+    V by = vfma(p3, uy, vfma(ph.a1, vfma(mphi, uy, h.y), tn * gr.y));
+    V bz = vfma(p3, uz, vfma(ph.a1, vfma(mphi, uz, h.z), tn * gr.z));
+    V a2 = ph.a2;
+    V e0 = al;
+    if constexpr (F16) {
+      const V k = vbc<V>(K);
+      bx = k * bx;
+      by = k * by;
+      bz = k * bz;
+      a2 = k * a2;
+      e0 = vfma(k, h.s - pc, al);  // phi of the cell is the shift of everything it writes
+    }
+    out.hrest(emit_rest<QH, F16>(h.s, e0));
+    emit_pairs<QH, F16>(h.s, e0, bx, by, bz, Gxx, Gyy, Gzz, a2 * h.xy, a2 * h.yz, a2 * h.xz,
+                        [&](int i, int oi, int cx, int cy, int cz, V A, V B) { out.h_(i, oi, cx, cy, cz, A, B); });
+  }
+}
+
+// w (s + r) for a lattice weight w, s the large part of a stored population
+// (phi or p*) and r the small rest.  FP32 carries w as hi + lo: the FP32
+// roundings of the D3Q15 weights alone sum to 1 + 7.5e-9 (D3Q27 likewise),
+// a bias of the zeroth and second moments that repeats every step and, over
+// 1000 steps, was the largest FP32 error of phi and u.
+__device__ __forceinline__ F1 wsum(double w, F1 s, F1 r) {
+  const float hi = (float)w, lo = (float)(w - (double)hi);
+  return vfma(F1{hi}, s, vfma(F1{lo}, s, F1{hi} * r));
+}
+
+// The collision of both sets in FP32, written around opposite-velocity pairs.
+// It keeps the operation order, each fused multiply-add included, that FP32 runs
+// have had throughout, so their results stay as they are: where the flow
+// amplifies FP32's rounding (the normal of a nearly uniform phi) another order
+// moves single cells by 1e-3 within 64 steps of a Taylor bubble, with no smaller
+// error against FP64.  The FP32 step is bound by memory, not by these operations.
+//   phi_at(cx, cy, cz): phi^t at a stencil neighbour; the rest as in collide().
+// FP32 and FP64 stores add the small terms first and the large part once.
+template <int QH, class PhiAt, class HM, class OUT>
+__device__ __forceinline__ void collide_pairs(const PhysR<float>& par, const PhiAt& phi_at, const Mom<F1>& gm, const HM& hmom,
+                                              OUT& out) {
+  typedef F1 V;
+  constexpr int QG = qg_of<QH>();   // D2Q9 with the 2-D phase field, else D3Q27
+  constexpr int GR = (QG - 1) / 2;  // rest index of g
+  const V third = vbc<V>(1.0 / 3.0), one = vbc<V>(1.0), half = vbc<V>(0.5), three = vbc<V>(3.0), k45 = vbc<V>(4.5),
+          zero = vbc<V>(0.0);
+  const V rho_l{par.rho_l}, drho{par.drho}, tau_l{par.tau_l}, dtau{par.dtau}, beta{par.beta}, kappa{par.kappa};
+
+  // ---- phi stencil over D3Q27 weights, by pairs
+  const V pc{phi_at(0, 0, 0)};
+  V gx = zero, gy = zero, gz = zero, lap = zero;
+#pragma unroll
+  for (int i = 0; i < GR; ++i) {
+    const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
+    const V a{phi_at(cx, cy, cz)}, b{phi_at(-cx, -cy, -cz)};
+    const V w = vbc<V>(lq_w<QG>(i)), d = a - b;
+    if (cx) gx = vfma(cx > 0 ? w : -w, d, gx);
+    if (cy) gy = vfma(cy > 0 ? w : -w, d, gy);
+    if (cz) gz = vfma(cz > 0 ? w : -w, d, gz);
+    lap = vfma(w, (a - pc) + (b - pc), lap);  // differences first: exact for nearby values
+  }
+  gx = gx * three;
+  gy = gy * three;
+  gz = gz * three;
+  lap = lap * vbc<V>(6.0);
+
+  // ---- forces and velocity
+  const V pst = gm.s;
+  const V rho = vfma(pc, drho, rho_l), tau = vfma(pc, dtau, tau_l);
+  const V omega = vrcp(tau);
+  const V nu = (tau - half) * third;
+  const V mu = vfma(((vbc<V>(4.0) * beta) * pc) * (pc - one), pc - half, -(kappa * lap));
+  const V inv2rho = vdiv(half, rho);
+  const V mc = vfma((-pst) * third, drho, mu);
+  V Fx = vfma(rho, V{par.gx}, mc * gx), Fy = vfma(rho, V{par.gy}, mc * gy), Fz = vfma(rho, V{par.gz}, mc * gz);
+  const V p3 = pst * third;
+  {
+    const V ax = vfma(Fx, inv2rho, gm.x), ay = vfma(Fy, inv2rho, gm.y), az = vfma(Fz, inv2rho, gm.z);
+    const V nxx = vfma(-ax, ax, gm.xx - p3), nyy = vfma(-ay, ay, gm.yy - p3), nzz = vfma(-az, az, gm.zz - p3);
+    const V nxy = vfma(-ax, ay, gm.xy), nyz = vfma(-ay, az, gm.yz), nxz = vfma(-ax, az, gm.xz);
+    const V cm = ((vbc<V>(-3.0) * nu) * omega) * drho;
+    Fx = vfma(cm, vfma(nxz, gz, vfma(nxx, gx, nxy * gy)), Fx);
+    Fy = vfma(cm, vfma(nyz, gz, vfma(nxy, gx, nyy * gy)), Fy);
+    Fz = vfma(cm, vfma(nzz, gz, vfma(nxz, gx, nyz * gy)), Fz);
+  }
+  const V ux = vfma(Fx, inv2rho, gm.x), uy = vfma(Fy, inv2rho, gm.y), uz = vfma(Fz, inv2rho, gm.z);
+
+  // ---- g post-collision coefficients and pair stores
+  {
+    const V x2 = ux * ux, y2 = uy * uy, z2 = uz * uz;
+    const V uu = (x2 + y2) + z2;
+    const V a2 = (one - omega) * k45;
+    // deviatoric second moments, (3 P_aa - p*) / 3 with one rounding: p* (1/3)
+    // would carry the rounded constant 1/3, a bias of 3e-8 p* that repeats
+    // every step
+    const V dxx = vfma(vfma(three, gm.xx, -pst), third, -x2), dyy = vfma(vfma(three, gm.yy, -pst), third, -y2);
+    const V dzz = QG == 9 ? zero : vfma(vfma(three, gm.zz, -pst), third, -z2);  // 2-D: the trace runs over x and y
+    const V als = vfma(vbc<V>(-1.5), uu, -((a2 * ((dxx + dyy) + dzz)) * third));
+    const V fr = vdiv(vbc<V>(1.5), rho);
+    const V bx = vfma(fr, Fx, three * ux), by = vfma(fr, Fy, three * uy), bz = vfma(fr, Fz, three * uz);
+    const V tx = k45 * ux, ty = k45 * uy, tz = k45 * uz;
+    const V Gxx = vfma(tx, ux, a2 * dxx), Gyy = vfma(ty, uy, a2 * dyy), Gzz = vfma(tz, uz, a2 * dzz);
+    const V two = vbc<V>(2.0);
+    const V Gxy = two * vfma(tx, uy, a2 * vfma(-ux, uy, gm.xy));
+    const V Gyz = two * vfma(ty, uz, a2 * vfma(-uy, uz, gm.yz));
+    const V Gxz = two * vfma(tx, uz, a2 * vfma(-ux, uz, gm.xz));
+    out.grest(wsum(lq_w<QG>(GR), pst, als));
+#pragma unroll
+    for (int i = 0; i < GR; ++i) {
+      const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
+      V E = zero, L = zero;
+      if (cx) E = E + Gxx;
+      if (cy) E = E + Gyy;
+      if (cz) E = E + Gzz;
+      if (cx && cy) E = E + ((cx * cy > 0) ? Gxy : -Gxy);
+      if (cy && cz) E = E + ((cy * cz > 0) ? Gyz : -Gyz);
+      if (cx && cz) E = E + ((cx * cz > 0) ? Gxz : -Gxz);
+      if (cx) L = L + (cx > 0 ? bx : -bx);
+      if (cy) L = L + (cy > 0 ? by : -by);
+      if (cz) L = L + (cz > 0 ? bz : -bz);
+      out.g_(i, QG - 1 - i, cx, cy, cz, wsum(lq_w<QG>(i), pst, als + (E + L)), wsum(lq_w<QG>(i), pst, als + (E - L)));
+    }
+  }
+
+  // ---- h post-collision coefficients and pair stores
+  {
+    const Mom<F1> h = hmom();
+    const V phl = h.s, omp{par.omega_phi};
+    const V gn = vsqrt(vfma(gz, gz, vfma(gy, gy, gx * gx)));
+    const V theta = ((vbc<V>(4.0) * pc) * (one - pc)) * V{par.inv_xi};
+    const V tn = vdiv(theta, gn + vbc<V>(1e-6)) * (one - half * omp);  // (1 - omega_phi/2) theta / |grad phi|
+    const V a1 = (one - omp) * three, a2 = (one - omp) * k45;
+    // deviatoric second moments as (3 H_aa - phi) / 3 and the non-equilibrium
+    // flux J - phi u, one rounding each
+    const V dxx = vfma(three, h.xx, -phl) * third, dyy = vfma(three, h.yy, -phl) * third;
+    const V dzz = QG == 9 ? zero : vfma(three, h.zz, -phl) * third;
+    const V als = ((-a2) * ((dxx + dyy) + dzz)) * third;
+    const V p3 = three * phl;
+    const V bx = vfma(tn, gx, vfma(p3, ux, a1 * vfma(-phl, ux, h.x)));
+    const V by = vfma(tn, gy, vfma(p3, uy, a1 * vfma(-phl, uy, h.y)));
+    const V bz = vfma(tn, gz, vfma(p3, uz, a1 * vfma(-phl, uz, h.z)));
+    const V a22 = vbc<V>(2.0) * a2;
+    out.hrest(wsum(hq_w<QH>(hq_rest<QH>()), phl, als));
+#pragma unroll
+    for (int k = 0; k < hq_rest<QH>(); ++k) {
+      const int cx = hq_cx<QH>(k), cy = hq_cy<QH>(k), cz = hq_cz<QH>(k);
+      V E = zero, L = zero;
+      if (cx) E = vfma(a2, dxx, E);
+      if (cy) E = vfma(a2, dyy, E);
+      if (cz) E = vfma(a2, dzz, E);
+      if (cx && cy) E = vfma((cx * cy > 0) ? a22 : -a22, h.xy, E);
+      if (cy && cz) E = vfma((cy * cz > 0) ? a22 : -a22, h.yz, E);
+      if (cx && cz) E = vfma((cx * cz > 0) ? a22 : -a22, h.xz, E);
+      if (cx) L = L + (cx > 0 ? bx : -bx);
+      if (cy) L = L + (cy > 0 ? by : -by);
+      if (cz) L = L + (cz > 0 ? bz : -bz);
+      out.h_(k, QH - 1 - k, cx, cy, cz, wsum(hq_w<QH>(k), phl, als + (E + L)), wsum(hq_w<QH>(k), phl, als + (E - L)));
+    }
+  }
+}
+
 // Store the post-collision pair (A: direction c, B: direction -c) of `cell`.
-template <int PREC, int ODD, class Off>
+template <int PREC, int ODD>
 __device__ __forceinline__ void store_pair(typename Store<PREC>::S* __restrict__ f, unsigned N, unsigned cell,
-                                           const Off& o, int i, int oi, int cx, int cy, int cz,
+                                           const CellOff& o, int i, int oi, int cx, int cy, int cz,
                                            typename Store<PREC>::R A, typename Store<PREC>::R B, Dither& d) {
   typename Store<PREC>::S a, b;
   if constexpr (PREC == 2 && PFL_FP16S_HWSR) {
@@ -338,348 +928,97 @@ __device__ __forceinline__ void store_pair(typename Store<PREC>::S* __restrict__
   }
 }
 
-// phi^t around a cell read from the current phi buffer (stencil offsets, so
-// mirrored across walls).
-template <int PREC>
-struct GlobalPhi {
-  const typename Store<PREC>::PhiT* __restrict__ phi;
-  const CellOff* o;
-  unsigned cell;
-  __device__ __forceinline__ typename Store<PREC>::R operator()(int cx, int cy, int cz) const {
-    return (typename Store<PREC>::R)__ldg(phi + cell + o->soff(cx, cy, cz));
-  }
-};
-
-// p* shift of the cell that wrote a g population (FP16S): the population
-// arriving from offset (dx, dy, dz) -- the opposite of its velocity -- was
-// written by `writer` (the neighbour, or the cell itself after a bounce-back,
-// valid = false).  GlobalShift reads the writer's shift from the per-cell
-// array; the fused step reads it from a shared-memory ring (SmemShift).
-struct GlobalShift {
-  const __half* __restrict__ p;
-  __device__ __forceinline__ float operator()(unsigned writer, int dx, int dy, int dz, bool valid) const {
-    return __half2float(__ldg(p + writer));
-  }
-};
-struct NoShift {
-  __device__ __forceinline__ float operator()(unsigned, int, int, int, bool) const { return 0.0f; }
-};
-
-// The collide-stream update of one cell, shared by every stream-collide
-// kernel: populations are read from (hin, gin) in the layout READ_ODD and
-// written to (hout, gout) in the layout WRITE_ODD (the same arrays and parity
-// for the in-place AA step; a second array pair and push streaming for the
-// two-array step).  phi_at(c) returns phi^t at the stencil neighbour c.
-template <int PREC, int QH, int READ_ODD, int WRITE_ODD, class PhiAt, int HM = 0, class PShift = NoShift,
-          class Off = CellOff>
-__device__ __forceinline__ void collide_cell(const Geo32& geo, const Phys& ph, const Off& o,
-                                             const typename Store<PREC>::S* hin,
-                                             const typename Store<PREC>::S* gin, typename Store<PREC>::S* hout,
-                                             typename Store<PREC>::S* gout, const PhiAt& phi_at,
-                                             const typename Store<PREC>::PhiT* __restrict__ shift,
-                                             unsigned cell, unsigned seed,
-                                             const typename Store<PREC>::R* hmom = nullptr, int hstride = 0,
-                                             const PShift& pshift = PShift(), __half* __restrict__ pg_out = nullptr) {
-  typedef typename Store<PREC>::R R;
-  constexpr bool F16 = PREC == 2;
-  constexpr int QG = qg_of<QH>();  // D2Q9 with the 2-D phase field, else D3Q27
-  constexpr int GR = (QG - 1) / 2;  // rest index of g
-  const unsigned N = geo.N;
-  Dither dith{F16 ? hash32(cell * 0x9E3779B1u + seed) : 0u};
-
-  // ---- phi stencil over D3Q27 weights, by pairs
-  const R pc = phi_at(0, 0, 0);
-  R gx = 0, gy = 0, gz = 0, lap = 0;
-#pragma unroll
-  for (int i = 0; i < GR; ++i) {
-    const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
-    const R a = phi_at(cx, cy, cz);
-    const R b = phi_at(-cx, -cy, -cz);
-    const R w = (R)lq_w<QG>(i);
-    const R d = w * (a - b);
-    if (cx) gx += cx > 0 ? d : -d;
-    if (cy) gy += cy > 0 ? d : -d;
-    if (cz) gz += cz > 0 ? d : -d;
-    lap += w * ((a - pc) + (b - pc));  // differences first: exact for nearby values
-  }
-  gx *= (R)3;
-  gy *= (R)3;
-  gz *= (R)3;
-  lap *= (R)6;
-
-  // ---- g moments (FP16: g_i = w_i (s / KG + P_writer))
-  R pst, jx = 0, jy = 0, jz = 0, pxx = 0, pyy = 0, pzz = 0, pxy = 0, pyz = 0, pxz = 0;
-  {
-    const R rest = raw<PREC>(gin[(unsigned)GR * N + cell]);
-    pst = F16 ? (rest * (R)(1.0 / KG16) + (R)pshift(cell, 0, 0, 0, false)) * (R)lq_w<QG>(GR) : rest;
-  }
-#pragma unroll
-  for (int i = 0; i < GR; ++i) {
-    const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
-    R a, b;
-    unsigned fa, fb;
-    load_pair<PREC, READ_ODD>(gin, N, cell, o, i, QG - 1 - i, cx, cy, cz, a, b, fa, fb);
-    R S = a + b, D = a - b;
-    if (F16) {
-      // a arrives from x - c, b from x + c
-      const R pa = (R)pshift(fa, -cx, -cy, -cz, o.valid(-cx, -cy, -cz));
-      const R pb = (R)pshift(fb, cx, cy, cz, o.valid(cx, cy, cz));
-      const R w = (R)lq_w<QG>(i);
-      S = w * (S * (R)(1.0 / KG16) + (pa + pb));
-      D = w * (D * (R)(1.0 / KG16) + (pa - pb));
-    }
-    pst += S;
-    if (cx) jx += cx > 0 ? D : -D;
-    if (cy) jy += cy > 0 ? D : -D;
-    if (cz) jz += cz > 0 ? D : -D;
-    if (cx) pxx += S;
-    if (cy) pyy += S;
-    if (cz) pzz += S;
-    if (cx && cy) pxy += (cx * cy > 0) ? S : -S;
-    if (cy && cz) pyz += (cy * cz > 0) ? S : -S;
-    if (cx && cz) pxz += (cx * cz > 0) ? S : -S;
-  }
-
-  // ---- forces and velocity (same expressions as hydro_macro)
-  const R drho = (R)(ph.rho_h - ph.rho_l);
-  const R rho = (R)ph.rho_l + pc * drho;
-  const R tau = (R)ph.tau_l + pc * (R)(ph.tau_h - ph.tau_l);
-  const R omega = (R)1 / tau;
-  const R nu = (tau - (R)0.5) * (R)(1.0 / 3.0);
-  const R mu = (R)4 * (R)ph.beta * pc * (pc - (R)1) * (pc - (R)0.5) - (R)ph.kappa * lap;
-  const R inv2rho = (R)0.5 / rho;
-  const R cp = -pst * (R)(1.0 / 3.0) * drho;
-  R Fx = (mu + cp) * gx + rho * (R)ph.gx;
-  R Fy = (mu + cp) * gy + rho * (R)ph.gy;
-  R Fz = (mu + cp) * gz + rho * (R)ph.gz;
-  const R p3 = pst * (R)(1.0 / 3.0);
-  {
-    const R u0x = jx + Fx * inv2rho, u0y = jy + Fy * inv2rho, u0z = jz + Fz * inv2rho;
-    const R nxx = pxx - p3 - u0x * u0x, nyy = pyy - p3 - u0y * u0y, nzz = pzz - p3 - u0z * u0z;
-    const R nxy = pxy - u0x * u0y, nyz = pyz - u0y * u0z, nxz = pxz - u0x * u0z;
-    const R cm = (R)-3 * nu * omega * drho;
-    Fx += cm * (nxx * gx + nxy * gy + nxz * gz);
-    Fy += cm * (nxy * gx + nyy * gy + nyz * gz);
-    Fz += cm * (nxz * gx + nyz * gy + nzz * gz);
-  }
-  const R ux = jx + Fx * inv2rho, uy = jy + Fy * inv2rho, uz = jz + Fz * inv2rho;
-  // FP16S: every g this cell writes is stored against P = fp16(p*) of the cell
-  R pw = 0;
-  if constexpr (F16) {
-    const __half q = __float2half_rn(pst);
-    pg_out[cell] = q;
-    pw = __half2float(q);
-  }
-
-  // ---- g post-collision coefficients and pair stores
-  {
-    const R uu = ux * ux + uy * uy + uz * uz;
-    const R a2 = ((R)1 - omega) * (R)4.5;
-    // deviatoric second moments.  FP32 / FP64 form (3 P_aa - p*) / 3 with one
-    // rounding: p* (1/3) would carry the rounded constant 1/3, a bias of
-    // 3e-8 p* that repeats every step (FP16S keeps its form)
-    const R third = (R)(1.0 / 3.0);
-    const R dxx = F16 ? pxx - p3 - ux * ux : fma((R)3, pxx, -pst) * third - ux * ux;
-    const R dyy = F16 ? pyy - p3 - uy * uy : fma((R)3, pyy, -pst) * third - uy * uy;
-    const R dzz = QG == 9 ? (R)0 : (F16 ? pzz - p3 - uz * uz : fma((R)3, pzz, -pst) * third - uz * uz);  // 2-D: the trace runs over x and y
-    const R K = F16 ? (R)KG16 : (R)1;
-    // alpha = p* + als with als small: FP32 and FP64 round p* once per stored
-    // value (FP16S stores K (alpha - P) + ... directly)
-    const R als = -(R)1.5 * uu - a2 * (dxx + dyy + dzz) * (R)(1.0 / 3.0);
-    const R al = K * (pst - pw - (R)1.5 * uu - a2 * (dxx + dyy + dzz) * (R)(1.0 / 3.0));
-    const R fr = (R)1.5 / rho;
-    const R bx = K * ((R)3 * ux + fr * Fx), by = K * ((R)3 * uy + fr * Fy), bz = K * ((R)3 * uz + fr * Fz);
-    const R Gxx = K * ((R)4.5 * ux * ux + a2 * dxx), Gyy = K * ((R)4.5 * uy * uy + a2 * dyy),
-            Gzz = K * ((R)4.5 * uz * uz + a2 * dzz);
-    const R Gxy = K * (R)2 * ((R)4.5 * ux * uy + a2 * (pxy - ux * uy));
-    const R Gyz = K * (R)2 * ((R)4.5 * uy * uz + a2 * (pyz - uy * uz));
-    const R Gxz = K * (R)2 * ((R)4.5 * ux * uz + a2 * (pxz - ux * uz));
-    gout[(unsigned)GR * N + cell] =
-        pack_sr<PREC>(F16 ? al : wsum<R>(lq_w<QG>(GR), pst, als), dith);
-#pragma unroll
-    for (int i = 0; i < GR; ++i) {
-      const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
-      // FP32 / FP64: the small terms first, the equilibrium part once (one
-      // rounding at its size); FP16S as E = al + ..., A = E + L
-      R E = F16 ? al : (R)0;
-      if (cx) E += Gxx;
-      if (cy) E += Gyy;
-      if (cz) E += Gzz;
-      if (cx && cy) E += (cx * cy > 0) ? Gxy : -Gxy;
-      if (cy && cz) E += (cy * cz > 0) ? Gyz : -Gyz;
-      if (cx && cz) E += (cx * cz > 0) ? Gxz : -Gxz;
-      R L = 0;
-      if (cx) L += cx > 0 ? bx : -bx;
-      if (cy) L += cy > 0 ? by : -by;
-      if (cz) L += cz > 0 ? bz : -bz;
-      R A, B;
-      if (F16) {
-        A = E + L;
-        B = E - L;
-      } else {
-        A = wsum<R>(lq_w<QG>(i), pst, als + (E + L));
-        B = wsum<R>(lq_w<QG>(i), pst, als + (E - L));
-      }
-      store_pair<PREC, WRITE_ODD>(gout, N, cell, o, i, QG - 1 - i, cx, cy, cz, A, B, dith);
-    }
-  }
-
-  // ---- h moments (shifted FP16: h = w (s / KH + phi_writer)), or given by the caller
-  R phl, hjx = 0, hjy = 0, hjz = 0, hxx = 0, hyy = 0, hzz = 0, hxy = 0, hyz = 0, hxz = 0;
-  if (HM) {
-    phl = hmom[0];
-    hjx = hmom[hstride];
-    hjy = hmom[2 * hstride];
-    hjz = hmom[3 * hstride];
-    hxx = hmom[4 * hstride];
-    hyy = hmom[5 * hstride];
-    hzz = hmom[6 * hstride];
-    hxy = hmom[7 * hstride];
-    hyz = hmom[8 * hstride];
-    hxz = hmom[9 * hstride];
-  } else {
-    const R rest = raw<PREC>(hin[(unsigned)hq_rest<QH>() * N + cell]);
-    phl = F16 ? (rest * (R)(1.0 / KH16) + (R)__ldg(shift + cell)) * (R)hq_w<QH>(hq_rest<QH>()) : rest;
-  }
-#pragma unroll
-  for (int k = 0; k < (HM ? 0 : hq_rest<QH>()); ++k) {
-    const int cx = hq_cx<QH>(k), cy = hq_cy<QH>(k), cz = hq_cz<QH>(k);
-    R a, b;
-    unsigned fa, fb;
-    load_pair<PREC, READ_ODD>(hin, N, cell, o, k, QH - 1 - k, cx, cy, cz, a, b, fa, fb);
-    R S, D;
-    if (F16) {
-      const R sa = (R)__ldg(shift + fa), sb = (R)__ldg(shift + fb);
-      const R w = (R)hq_w<QH>(k);
-      S = w * ((a + b) * (R)(1.0 / KH16) + (sa + sb));
-      D = w * ((a - b) * (R)(1.0 / KH16) + (sa - sb));
-    } else {
-      S = a + b;
-      D = a - b;
-    }
-    phl += S;
-    if (cx) hjx += cx > 0 ? D : -D;
-    if (cy) hjy += cy > 0 ? D : -D;
-    if (cz) hjz += cz > 0 ? D : -D;
-    if (cx) hxx += S;
-    if (cy) hyy += S;
-    if (cz) hzz += S;
-    if (cx && cy) hxy += (cx * cy > 0) ? S : -S;
-    if (cy && cz) hyz += (cy * cz > 0) ? S : -S;
-    if (cx && cz) hxz += (cx * cz > 0) ? S : -S;
-  }
-
-  // ---- h post-collision coefficients and pair stores
-  {
-    const R omp = (R)ph.omega_phi;
-    const R gn = sqrt(gx * gx + gy * gy + gz * gz);
-    const R theta = (R)4 * pc * ((R)1 - pc) * (R)ph.inv_xi;
-    const R tn = theta / (gn + (R)1e-6) * ((R)1 - (R)0.5 * omp);  // (1 - omega_phi/2) theta / |grad phi|
-    const R a1 = ((R)1 - omp) * (R)3, a2 = ((R)1 - omp) * (R)4.5;
-    // deviatoric second moments and the non-equilibrium flux.  FP32 / FP64
-    // form (3 H_aa - phi) / 3 and J - phi u with one rounding each: phi (1/3)
-    // would carry the rounded constant 1/3, a bias of 3e-8 phi that repeats
-    // every step (FP16S keeps its form)
-    const R ph3 = phl * (R)(1.0 / 3.0);
-    const R third = (R)(1.0 / 3.0);
-    const R dxx = F16 ? hxx - ph3 : fma((R)3, hxx, -phl) * third;
-    const R dyy = F16 ? hyy - ph3 : fma((R)3, hyy, -phl) * third;
-    const R dzz = QG == 9 ? (R)0 : (F16 ? hzz - ph3 : fma((R)3, hzz, -phl) * third);
-    const R K = F16 ? (R)KH16 : (R)1;
-    const R sh = F16 ? pc : (R)0;   // this cell's phi: the shift of everything it writes
-    // alpha = phi + als with als small: FP32 and FP64 round phi once per stored
-    // value (FP16S stores K (alpha - phi_x) + ... directly)
-    const R als = -a2 * (dxx + dyy + dzz) * (R)(1.0 / 3.0);
-    const R al = K * ((phl - sh) - a2 * (dxx + dyy + dzz) * (R)(1.0 / 3.0));
-    const R jdx = F16 ? hjx - phl * ux : fma(-phl, ux, hjx);
-    const R jdy = F16 ? hjy - phl * uy : fma(-phl, uy, hjy);
-    const R jdz = F16 ? hjz - phl * uz : fma(-phl, uz, hjz);
-    const R bx = K * ((R)3 * phl * ux + a1 * jdx + tn * gx);
-    const R by = K * ((R)3 * phl * uy + a1 * jdy + tn * gy);
-    const R bz = K * ((R)3 * phl * uz + a1 * jdz + tn * gz);
-    const R Gxx = K * a2 * dxx, Gyy = K * a2 * dyy, Gzz = K * a2 * dzz;
-    const R Gxy = K * (R)2 * a2 * hxy, Gyz = K * (R)2 * a2 * hyz, Gxz = K * (R)2 * a2 * hxz;
-    hout[(unsigned)hq_rest<QH>() * N + cell] =
-        pack_sr<PREC>(F16 ? al : wsum<R>(hq_w<QH>(hq_rest<QH>()), phl, als), dith);
-#pragma unroll
-    for (int k = 0; k < hq_rest<QH>(); ++k) {
-      const int cx = hq_cx<QH>(k), cy = hq_cy<QH>(k), cz = hq_cz<QH>(k);
-      R E = F16 ? al : (R)0;
-      if (cx) E += Gxx;
-      if (cy) E += Gyy;
-      if (cz) E += Gzz;
-      if (cx && cy) E += (cx * cy > 0) ? Gxy : -Gxy;
-      if (cy && cz) E += (cy * cz > 0) ? Gyz : -Gyz;
-      if (cx && cz) E += (cx * cz > 0) ? Gxz : -Gxz;
-      R L = 0;
-      if (cx) L += cx > 0 ? bx : -bx;
-      if (cy) L += cy > 0 ? by : -by;
-      if (cz) L += cz > 0 ? bz : -bz;
-      R A, B;
-      if (F16) {
-        A = E + L;
-        B = E - L;
-      } else {
-        A = wsum<R>(hq_w<QH>(k), phl, als + (E + L));
-        B = wsum<R>(hq_w<QH>(k), phl, als + (E - L));
-      }
-      store_pair<PREC, WRITE_ODD>(hout, N, cell, o, k, QH - 1 - k, cx, cy, cz, A, B, dith);
-    }
-  }
+// Stored value of direction c arriving at `cell`, raw; `from` the cell that
+// wrote it.  READ_ODD: the state left by an even in-place step.
+template <int PREC, int Q, int READ_ODD>
+__device__ __forceinline__ typename Store<PREC>::R load_dir(const typename Store<PREC>::S* f, unsigned N, unsigned cell,
+                                                            const CellOff& o, int cx, int cy, int cz) {
+  const int i = lq_index<Q>(cx, cy, cz);
+  if (!READ_ODD || (!cx && !cy && !cz)) return raw<PREC>(f[(unsigned)i * N + cell]);
+  const bool v = o.valid(-cx, -cy, -cz);
+  return raw<PREC>(f[v ? (unsigned)(Q - 1 - i) * N + cell + (unsigned)o.off(-cx, -cy, -cz) : (unsigned)i * N + cell]);
 }
+// the cell that wrote the population of direction c arriving at `cell`
+__device__ __forceinline__ unsigned writer(unsigned cell, const CellOff& o, int cx, int cy, int cz) {
+  return o.valid(-cx, -cy, -cz) ? cell + (unsigned)o.off(-cx, -cy, -cz) : cell;
+}
+
+// The h moments of one cell of a state in memory.
+template <int PREC, int QH, int READ_ODD>
+__device__ __forceinline__ Mom<typename StepV<PREC>::T> h_moments_cell(
+    unsigned N, const typename Store<PREC>::S* h, const typename Store<PREC>::PhiT* __restrict__ shift, unsigned cell,
+    const CellOff& o) {
+  typedef typename StepV<PREC>::T V;
+  return h_moments<PREC, QH, V>(
+      [&](int cx, int cy, int cz) { return V{load_dir<PREC, QH, READ_ODD>(h, N, cell, o, cx, cy, cz)}; },
+      [&](int cx, int cy, int cz) { return V{(typename V::R)__ldg(shift + writer(cell, o, cx, cy, cz))}; });
+}
+
+// Destination of one cell's collision: the pairs go to (h, g) in the layout
+// ODD; FP16S: its p* shift to pg_out.
+template <int PREC, int QH, int ODD>
+struct CellOut {
+  typedef typename StepV<PREC>::T V;
+  typename Store<PREC>::S *h, *g;
+  unsigned N, cell;
+  const CellOff& o;
+  __half* pg_out;
+  Dither dith;
+  __device__ __forceinline__ V shift(V pst) {
+    const __half q = __float2half_rn((float)pst.v);
+    pg_out[cell] = q;
+    return V{(typename V::R)__half2float(q)};
+  }
+  __device__ __forceinline__ void grest(V v) { g[(unsigned)((qg_of<QH>() - 1) / 2) * N + cell] = pack_sr<PREC>(v.v, dith); }
+  __device__ __forceinline__ void hrest(V v) { h[(unsigned)hq_rest<QH>() * N + cell] = pack_sr<PREC>(v.v, dith); }
+  __device__ __forceinline__ void g_(int i, int oi, int cx, int cy, int cz, V A, V B) {
+    store_pair<PREC, ODD>(g, N, cell, o, i, oi, cx, cy, cz, A.v, B.v, dith);
+  }
+  __device__ __forceinline__ void h_(int i, int oi, int cx, int cy, int cz, V A, V B) {
+    store_pair<PREC, ODD>(h, N, cell, o, i, oi, cx, cy, cz, A.v, B.v, dith);
+  }
+};
 
 // In-place AA update of one cell with the stencil read from the phi buffer.
 // pg_in / pg_out: the p* shifts of the stored g (FP16S; NULL otherwise),
 // read for the populations loaded and written for those stored.
 template <int PREC, int QH, int ODD>
-__device__ __forceinline__ void step_cell(const Geo32& geo, const Phys& ph, typename Store<PREC>::S* __restrict__ h,
+__device__ __forceinline__ void step_cell(const Geo32& geo, const typename StepV<PREC>::Par& ph,
+                                          typename Store<PREC>::S* __restrict__ h,
                                           typename Store<PREC>::S* __restrict__ g,
                                           const typename Store<PREC>::PhiT* __restrict__ phi,
                                           const typename Store<PREC>::PhiT* __restrict__ shift, unsigned cell,
-                                          unsigned seed, const __half* __restrict__ pg_in = nullptr,
-                                          __half* __restrict__ pg_out = nullptr) {
+                                          unsigned seed, const __half* __restrict__ pg_in, __half* __restrict__ pg_out) {
+  typedef typename StepV<PREC>::T V;
+  typedef typename V::R R;
+  constexpr int QG = qg_of<QH>();
   CellOff o;
   cell_off(geo, cell, o);
-  GlobalPhi<PREC> at{phi, &o, cell};
-  collide_cell<PREC, QH, ODD, ODD, GlobalPhi<PREC>, 0, GlobalShift>(geo, ph, o, h, g, h, g, at, shift, cell, seed,
-                                                                    nullptr, 0, GlobalShift{pg_in}, pg_out);
+  auto at = [&](int cx, int cy, int cz) { return (R)__ldg(phi + cell + o.soff(cx, cy, cz)); };
+  const Mom<V> gm = g_moments<PREC, QG, V>(
+      [&](int cx, int cy, int cz) { return V{load_dir<PREC, QG, ODD>(g, geo.N, cell, o, cx, cy, cz)}; },
+      [&](int cx, int cy, int cz) { return V{(R)__half2float(__ldg(pg_in + writer(cell, o, cx, cy, cz)))}; });
+  CellOut<PREC, QH, ODD> out{h, g, geo.N, cell, o, pg_out, Dither{PREC == 2 ? hash32(cell * 0x9E3779B1u + seed) : 0u}};
+  auto hm = [&] { return h_moments_cell<PREC, QH, ODD>(geo.N, h, shift, cell, o); };
+  if constexpr (PREC == 1) {
+    collide_pairs<QH>(ph, at, gm, hm, out);
+  } else {
+    auto plane = [&](int cz) { return phi_plane<V>([&](int cx, int cy) { return V{at(cx, cy, cz)}; }); };
+    const PhiPlane<V> p0 = plane(0);
+    const Grad<V> gr = QG == 9 ? phi_grad_flat(p0) : phi_grad(plane(-1), p0, plane(1));
+    collide<PREC, QH, V>(ph, p0.c, gr, gm, hm, out);
+  }
 }
 
 template <int PREC, int QH, int ODD>
 __global__ void __launch_bounds__(PFL_STEP_THREADS, PFL_STEP_MINB)
-    k_step_mrt(Geo32 geo, Phys ph, typename Store<PREC>::S* __restrict__ h, typename Store<PREC>::S* __restrict__ g,
-               const typename Store<PREC>::PhiT* __restrict__ phi,
+    k_step_mrt(Geo32 geo, typename StepV<PREC>::Par ph, typename Store<PREC>::S* __restrict__ h,
+               typename Store<PREC>::S* __restrict__ g, const typename Store<PREC>::PhiT* __restrict__ phi,
                const typename Store<PREC>::PhiT* __restrict__ shift, unsigned seed,
                const __half* __restrict__ pg_in = nullptr, __half* __restrict__ pg_out = nullptr) {
   const unsigned cell = blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= geo.N) return;
   step_cell<PREC, QH, ODD>(geo, ph, h, g, phi, shift, cell, seed, pg_in, pg_out);
-}
-
-// phi of one cell from the stored h (READ_ODD after an even step).
-template <int PREC, int QH, int READ_ODD>
-__device__ __forceinline__ typename Store<PREC>::R phi_cell(const Geo32& geo,
-                                                            const typename Store<PREC>::S* __restrict__ h,
-                                                            const typename Store<PREC>::PhiT* __restrict__ shift,
-                                                            unsigned cell, unsigned blk = 0) {
-  typedef typename Store<PREC>::R R;
-  constexpr bool F16 = PREC == 2;
-  CellOff o;
-  cell_off(geo, cell, o);
-  o.blk = blk;  // a bounced population was written by this cell
-  R s = F16 ? (raw<PREC>(h[(unsigned)hq_rest<QH>() * geo.N + cell]) * (R)(1.0 / KH16) + (R)__ldg(shift + cell)) * (R)hq_w<QH>(hq_rest<QH>())
-            : raw<PREC>(h[(unsigned)hq_rest<QH>() * geo.N + cell]);
-#pragma unroll
-  for (int k = 0; k < hq_rest<QH>(); ++k) {
-    R a, b;
-    unsigned fa, fb;
-    load_pair<PREC, READ_ODD>(h, geo.N, cell, o, k, QH - 1 - k, hq_cx<QH>(k), hq_cy<QH>(k), hq_cz<QH>(k), a, b, fa, fb);
-    if (F16)
-      s += (R)hq_w<QH>(k) * ((a + b) * (R)(1.0 / KH16) + ((R)__ldg(shift + fa) + (R)__ldg(shift + fb)));
-    else
-      s += a + b;
-  }
-  return s;
 }
 
 // phi = sum_i h_i of the state left by the last step (READ_ODD after an even
@@ -691,15 +1030,14 @@ __global__ void __launch_bounds__(256) k_phi32(Geo32 geo, const typename Store<P
                                                const typename Store<PREC>::PhiT* __restrict__ shift,
                                                typename Store<PREC>::PhiT* __restrict__ phi,
                                                const unsigned* __restrict__ links = nullptr) {
+  typedef typename Store<PREC>::PhiT PhiT;
   const unsigned cell = blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= geo.N) return;
-  const unsigned blk = links ? __ldg(links + cell) : 0u;
-  phi[cell] = (blk & SOLID_SELF) ? (typename Store<PREC>::PhiT)0 : phi_cell<PREC, QH, READ_ODD>(geo, h, shift, cell, blk);
+  CellOff o;
+  cell_off(geo, cell, o);
+  o.blk = links ? __ldg(links + cell) : 0u;  // a bounced population was written by this cell
+  phi[cell] = (o.blk & SOLID_SELF) ? (PhiT)0 : (PhiT)h_moments_cell<PREC, QH, READ_ODD>(geo.N, h, shift, cell, o).s.v;
 }
-
-}  // namespace pfl
-
-namespace pfl {
 
 // ---------------------------------------------------------------------------
 // Fused two-array step: stream-collide and the phi stencil in one launch.
@@ -708,13 +1046,13 @@ namespace pfl {
 // its own cell (every slot local, coalesced) and pushes the post-collision
 // populations to the other pair (x + c, or the opposite slot of x behind a
 // wall).  Nothing a step reads is overwritten during that step, so a block may
-// read its neighbours' populations: each block owns an xy tile of ZM_TX x
-// ZM_TY columns and marches through a chunk of z planes, computing phi^t =
-// sum_i h_i for its tile plus a one-cell ring into a three-plane shared-memory
-// ring before colliding a plane.  phi^t of every cell is written once (the
-// FP16S shift of the populations written this step and the phi output), so
-// the separate phi pass and its re-read of h disappear.  Ring and z-halo
-// planes repeat the phi sum of neighbouring tiles (from L2).
+// read its neighbours' populations: each block owns an xy tile of TX x TY
+// columns and marches through a chunk of z planes, computing phi^t = sum_i h_i
+// for its tile plus a one-cell ring of the next plane into shared memory before
+// colliding a plane.  phi^t of every cell is written once (the FP16S shift of
+// the populations written this step and the phi output), so the separate phi
+// pass and its re-read of h disappear.  Ring and z-halo planes repeat the phi
+// sum of neighbouring tiles (from L2).
 // A single-plane lattice (FLAT) has no z march to hide latency behind; its
 // tiles are 32 x 4, so that a small lattice spreads over more blocks (and the
 // SMs' loads even out) for a slightly larger share of ring cells.
@@ -722,157 +1060,21 @@ constexpr int ZM_TX = 32;
 constexpr int ZM_TY = 8;
 constexpr int ZM_TY_FLAT = 4;
 __host__ __device__ constexpr int zm_ty(int flat) { return flat ? ZM_TY_FLAT : ZM_TY; }
-
-// FLAT: a single plane, its own z neighbour (periodic) -- every cz reads the
-// plane itself, so the compiler loads each in-plane value once.
-template <int PREC, int FLAT = 0, int PW = ZM_TX + 2>
-struct SmemPhi {
-  const typename Store<PREC>::PhiT* plane[3];  // planes z - 1, z, z + 1 of (tile height + 2) x PW values
-  int i0;                 // index of this thread's column in a plane
-  unsigned blk = 0;       // blocked links: a solid neighbour reads as this cell (neutral wetting)
-  __device__ __forceinline__ typename Store<PREC>::R operator()(int cx, int cy, int cz) const {
-    if (blk & link_bit(cx, cy, cz)) return (typename Store<PREC>::R)plane[1][i0];
-    return (typename Store<PREC>::R)plane[FLAT ? 1 : 1 + cz][i0 + cy * PW + cx];
-  }
-};
-
-// p* shift of the writer of a g population from the ring of P planes z - 1,
-// z, z + 1 of the fused step (tile plus a one-cell ring, like SmemPhi): the
-// neighbour at (dx, dy, dz), or the cell itself after a bounce-back.
-template <int FLAT = 0, int PW = ZM_TX + 2>
-struct SmemShift {
-  const float* plane[3];
-  int i0;
-  __device__ __forceinline__ float operator()(unsigned, int dx, int dy, int dz, bool valid) const {
-    return valid ? plane[FLAT ? 1 : 1 + dz][i0 + dy * PW + dx] : plane[1][i0];
-  }
-};
+// resident blocks per SM a block of nt threads is compiled for
+__host__ __device__ constexpr int zm_minb(int prec, int nt) {
+  return (prec == 0 ? PFL_ZM_MINB_FP64 : PFL_ZM_MINB) * 256 / nt;
+}
 
 __device__ __forceinline__ void prefetch_l1(const void* p) {
   asm volatile("{\n\t.reg .u64 ga;\n\tcvta.to.global.u64 ga, %0;\n\tprefetch.global.L1 [ga];\n\t}" ::"l"(p));
 }
 
+// v one step outside [0, n) brought inside (wrapped, or clamped at walls);
+// positions further out, which nothing uses, to the last cell
 __device__ __forceinline__ int wrap_or_clamp(int v, int n, int wall) {
-  if (wall) return v < 0 ? 0 : (v >= n ? n - 1 : v);
-  return v < 0 ? v + n : (v >= n ? v - n : v);
-}
-
-// The 10 h moments (phi, sum c h, sum c c h) of `cell` of the current pair
-// (normal layout, neighbour offsets o), accumulated by pairs in the same order
-// as the collision does, so moms[0] equals its phi bitwise.
-template <int PREC, int QH, class Off>
-__device__ __forceinline__ void h_moments_at(const Geo32& geo, const typename Store<PREC>::S* __restrict__ h,
-                                             const typename Store<PREC>::PhiT* __restrict__ shift, unsigned cell,
-                                             const Off& o, typename Store<PREC>::R m[10]) {
-  typedef typename Store<PREC>::R R;
-  constexpr bool F16 = PREC == 2;
-  const unsigned N = geo.N;
-  R phl, hjx = 0, hjy = 0, hjz = 0, hxx = 0, hyy = 0, hzz = 0, hxy = 0, hyz = 0, hxz = 0;
-  {
-    const R rest = raw<PREC>(h[(unsigned)hq_rest<QH>() * N + cell]);
-    phl = F16 ? (rest * (R)(1.0 / KH16) + (R)__ldg(shift + cell)) * (R)hq_w<QH>(hq_rest<QH>()) : rest;
-  }
-#pragma unroll
-  for (int k = 0; k < hq_rest<QH>(); ++k) {
-    const int cx = hq_cx<QH>(k), cy = hq_cy<QH>(k), cz = hq_cz<QH>(k);
-    R a, b;
-    unsigned fa, fb;
-    load_pair<PREC, 0>(h, N, cell, o, k, QH - 1 - k, cx, cy, cz, a, b, fa, fb);
-    R S, D;
-    if (F16) {
-      const R sa = (R)__ldg(shift + fa), sb = (R)__ldg(shift + fb);
-      const R w = (R)hq_w<QH>(k);
-      S = w * ((a + b) * (R)(1.0 / KH16) + (sa + sb));
-      D = w * ((a - b) * (R)(1.0 / KH16) + (sa - sb));
-    } else {
-      S = a + b;
-      D = a - b;
-    }
-    phl += S;
-    if (cx) hjx += cx > 0 ? D : -D;
-    if (cy) hjy += cy > 0 ? D : -D;
-    if (cz) hjz += cz > 0 ? D : -D;
-    if (cx) hxx += S;
-    if (cy) hyy += S;
-    if (cz) hzz += S;
-    if (cx && cy) hxy += (cx * cy > 0) ? S : -S;
-    if (cy && cz) hyz += (cy * cz > 0) ? S : -S;
-    if (cx && cz) hxz += (cx * cz > 0) ? S : -S;
-  }
-  m[0] = phl;
-  m[1] = hjx;
-  m[2] = hjy;
-  m[3] = hjz;
-  m[4] = hxx;
-  m[5] = hyy;
-  m[6] = hzz;
-  m[7] = hxy;
-  m[8] = hyz;
-  m[9] = hxz;
-}
-
-// phi of `cell` of the current pair (normal layout), same sum as the phi pass.
-template <int PREC, int QH, class Off>
-__device__ __forceinline__ typename Store<PREC>::R phi_at(const Geo32& geo, const typename Store<PREC>::S* __restrict__ h,
-                                                          const typename Store<PREC>::PhiT* __restrict__ shift,
-                                                          unsigned cell, const Off& o) {
-  typedef typename Store<PREC>::R R;
-  constexpr bool F16 = PREC == 2;
-  R s = F16 ? (raw<PREC>(h[(unsigned)hq_rest<QH>() * geo.N + cell]) * (R)(1.0 / KH16) + (R)__ldg(shift + cell)) * (R)hq_w<QH>(hq_rest<QH>())
-            : raw<PREC>(h[(unsigned)hq_rest<QH>() * geo.N + cell]);
-#pragma unroll
-  for (int k = 0; k < hq_rest<QH>(); ++k) {
-    R a, b;
-    unsigned fa, fb;
-    load_pair<PREC, 0>(h, geo.N, cell, o, k, QH - 1 - k, hq_cx<QH>(k), hq_cy<QH>(k), hq_cz<QH>(k), a, b, fa, fb);
-    if (F16)
-      s += (R)hq_w<QH>(k) * ((a + b) * (R)(1.0 / KH16) + ((R)__ldg(shift + fa) + (R)__ldg(shift + fb)));
-    else
-      s += a + b;
-  }
-  return s;
-}
-
-// Offsets of cell (x, y, z): the general form, or (INT) the interior one.
-template <int INT>
-struct OffOf;
-template <>
-struct OffOf<0> {
-  typedef CellOff T;
-  static __device__ __forceinline__ CellOff at(const Geo32& geo, unsigned x, unsigned y, unsigned z, unsigned blk) {
-    CellOff o;
-    o.X = axis_off(x, geo.nx, 1, geo.wall[0]);
-    o.Y = axis_off(y, geo.ny, (int)geo.nx, geo.wall[1]);
-    o.Z = axis_off(z, geo.nz, (int)(geo.nx * geo.ny), geo.wall[2]);
-    o.blk = blk;  // a bounced population was written by this cell
-    return o;
-  }
-};
-template <>
-struct OffOf<1> {
-  typedef CellOffI T;
-  static __device__ __forceinline__ CellOffI at(const Geo32& geo, unsigned, unsigned, unsigned, unsigned) {
-    return CellOffI{(int)geo.nx, geo.nz == 1 ? 0 : (int)(geo.nx * geo.ny)};
-  }
-};
-
-template <int PREC, int QH, int INT = 0>
-__device__ __forceinline__ void h_moments_xyz(const Geo32& geo, const typename Store<PREC>::S* __restrict__ h,
-                                              const typename Store<PREC>::PhiT* __restrict__ shift, unsigned x,
-                                              unsigned y, unsigned z, typename Store<PREC>::R m[10],
-                                              unsigned blk = 0) {
-  const unsigned cell = x + geo.nx * (y + geo.ny * z);
-  h_moments_at<PREC, QH>(geo, h, shift, cell, OffOf<INT>::at(geo, x, y, z, blk), m);
-}
-
-template <int PREC, int QH, int INT = 0>
-__device__ __forceinline__ typename Store<PREC>::R phi_at_xyz(const Geo32& geo,
-                                                              const typename Store<PREC>::S* __restrict__ h,
-                                                              const typename Store<PREC>::PhiT* __restrict__ shift,
-                                                              unsigned x, unsigned y, unsigned z,
-                                                              unsigned blk = 0) {
-  const unsigned cell = x + geo.nx * (y + geo.ny * z);
-  return phi_at<PREC, QH>(geo, h, shift, cell, OffOf<INT>::at(geo, x, y, z, blk));
+  if (v < 0) return wall ? 0 : n - 1;
+  if (v < n) return v;
+  return wall ? n - 1 : min(v - n, n - 1);
 }
 
 // position r in [0, 2 (W + H) - 4) of the frame of a W x H plane -> (i, j)
@@ -892,18 +1094,23 @@ __device__ __forceinline__ void frame_pos(int r, int W, int H, int& i, int& j) {
   }
 }
 
-// grid: (ceil(nx / ZM_TX), ceil(ny / TY), ceil(nz / zc)), block ZM_TX x TY with
-// TY = zm_ty(FLAT).
-// SOLID: the lattice holds solid cells, given by `links` (one word per cell).
-// tclock (launches replayed from a CUDA graph): the FP16 rounding seed comes
-// from the step count *tclock + tofs in device memory instead of `seed`, the
-// same function of the step count as the host's.
+__device__ __forceinline__ CellOff off_xyz(const Geo32& geo, unsigned x, unsigned y, unsigned z, unsigned blk) {
+  CellOff o;
+  o.X = axis_off(x, geo.nx, 1, geo.wall[0]);
+  o.Y = axis_off(y, geo.ny, (int)geo.nx, geo.wall[1]);
+  o.Z = axis_off(z, geo.nz, (int)(geo.nx * geo.ny), geo.wall[2]);
+  o.blk = blk;
+  return o;
+}
+
 // One tile of the fused step: the xy tile (bx, by) of TX x TY columns and
 // the z chunk bz of zc planes (the grid of k_step_zm, or an entry of the
 // batched engine's work list), run by a block of TX x TY threads.  The caller
-// has waited for the previous step.
+// has waited for the previous step.  SOLID: the lattice holds solid cells, given
+// by `links` (one word per cell).
 template <int PREC, int QH, int TY, int FLAT, int SOLID, int TX = ZM_TX>
-__device__ __forceinline__ void zm_tile(const Geo32& geo, const Phys& ph, const typename Store<PREC>::S* __restrict__ hA,
+__device__ __forceinline__ void zm_tile(const Geo32& geo, const typename StepV<PREC>::Par& ph,
+                                        const typename Store<PREC>::S* __restrict__ hA,
                                         const typename Store<PREC>::S* __restrict__ gA,
                                         typename Store<PREC>::S* __restrict__ hB, typename Store<PREC>::S* __restrict__ gB,
                                         const typename Store<PREC>::PhiT* __restrict__ phi_shift,
@@ -911,125 +1118,173 @@ __device__ __forceinline__ void zm_tile(const Geo32& geo, const Phys& ph, const 
                                         const unsigned* __restrict__ links, const __half* __restrict__ pg_in,
                                         __half* __restrict__ pg_out, int bx, int by, int bz) {
   typedef typename Store<PREC>::PhiT PhiT;
+  typedef typename Store<PREC>::S S;
   typedef typename Store<PREC>::R R;
+  typedef typename StepV<PREC>::T V;
   constexpr int NT = TX * TY;
   constexpr int PW = TX + 2, PH = TY + 2, PS = PW * PH;
   constexpr int NRING = 2 * (PW + PH) - 4;
-  static_assert(NRING <= NT, "one thread per ring position");
-  // phi planes z - 1, z, z + 1 and the one being filled: with four slots the
-  // fill of plane z + 1 overwrites plane z - 3, which every thread finished
-  // reading before the barrier of the previous plane, so one barrier per plane
-  // suffices.  The h moments are per thread and need none.  FP64 keeps three
-  // slots (static shared memory stays under 48 KB) and a second barrier.
-  constexpr int NS = FLAT ? 1 : (sizeof(R) == 8 ? 3 : 4);
-  __shared__ PhiT ring[NS][PS];
-  __shared__ R hmom[FLAT ? 1 : 2][10 * NT];  // h moments of the tile's own cells
   constexpr bool F16 = PREC == 2;
-  __shared__ float pring[F16 ? NS : 1][F16 ? PS : 1];  // FP16S: p* shifts of the stored g, ring like phi
+  constexpr int QG = qg_of<QH>();
+  // phi planes.  MARCH: the one being filled and the one being read, whose
+  // in-plane stencil part is kept in registers (two slots, one barrier per
+  // plane: a slot is refilled only after the barrier that follows its last
+  // read).  FP32, and solid cells, whose stencil reads depend on the reading
+  // cell: all three planes of the stencil and the one being filled (FP64: three
+  // slots, within 48 KB of static shared memory, and a second barrier).  The p*
+  // shifts are read for three planes as well.  The h moments are per thread.
+  constexpr bool MARCH = PREC != 1 && !SOLID;
+  constexpr int NS = FLAT ? 1 : (MARCH ? 2 : (sizeof(R) == 8 ? 3 : 4));
+  constexpr int NSP = FLAT ? 1 : 4;
+  __shared__ PhiT ring[NS][PS];
+  __shared__ V hmom[FLAT ? 1 : 2][10 * NT];
+  __shared__ float pring[F16 ? NSP : 1][F16 ? PS : 1];  // FP16S: p* shifts of the stored g, ring like phi
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
   const int x0 = bx * TX, y0 = by * TY;
   const int z0 = bz * zc;
   const int z1 = min(z0 + zc, (int)geo.nz);
+  const unsigned N = geo.N;
   const int x = x0 + tx, y = y0 + ty;
   const bool active = x < (int)geo.nx && y < (int)geo.ny;
+  const int i0 = (ty + 1) * PW + tx + 1;  // ring position of the own cell
   const unsigned xq = (unsigned)wrap_or_clamp(x, (int)geo.nx, geo.wall[0]);
   const unsigned yq = (unsigned)wrap_or_clamp(y, (int)geo.ny, geo.wall[1]);
-  int ri = 0, rj = 0;
-  if (tid < NRING) frame_pos(tid, PW, PH, ri, rj);
-  const unsigned rxq = (unsigned)wrap_or_clamp(x0 - 1 + ri, (int)geo.nx, geo.wall[0]);
-  const unsigned ryq = (unsigned)wrap_or_clamp(y0 - 1 + rj, (int)geo.ny, geo.wall[1]);
 
   // L1 prefetch of the g populations plane zp's collision will read
   auto prefetch_plane = [&](int zp) {
     if (!(PFL_ZM_PREFETCH && PREC == 1 && QH == 15 && !FLAT) || !active || zp >= z1) return;
-    constexpr int QG = qg_of<QH>();
     const unsigned c = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)zp);
 #pragma unroll
-    for (int i = 0; i < QG; ++i) prefetch_l1(gA + (unsigned)i * geo.N + c);
+    for (int i = 0; i < QG; ++i) prefetch_l1(gA + (unsigned)i * N + c);
   };
-
-  // The march over the block's z planes, in the general form (INT = 0) or, for
-  // blocks whose tile, ring and planes z0 - 2 .. z1 + 1 lie clear of the
-  // lattice's faces, the interior one (INT = 1: every link valid, neighbour
-  // offsets without wall or wrap tests).
-  auto march = [&](auto int_tag) {
-  constexpr int INT = decltype(int_tag)::value;
+  // phi of cell (qx, qy, zq) from memory
+  auto phi_at = [&](unsigned qx, unsigned qy, unsigned zq) {
+    const unsigned c = qx + geo.nx * (qy + geo.ny * zq);
+    CellOff o;
+    if (F16) o = off_xyz(geo, qx, qy, zq, SOLID ? __ldg(links + c) : 0u);
+    return (PhiT)h_moments_cell<PREC, QH, 0>(N, hA, phi_shift, c, o).s.v;
+  };
   // phi of plane zp over the tile (with the h moments of the own cells) and its ring
-  auto fill = [&](int zp, int slot, int mslot) {
+  auto fill = [&](int zp, int slot, int pslot, int mslot) {
     const unsigned zq = (unsigned)wrap_or_clamp(zp, (int)geo.nz, geo.wall[2]);
-    R m[10];
-    const unsigned bt = SOLID ? __ldg(links + xq + geo.nx * (yq + geo.ny * zq)) : 0u;
-    h_moments_xyz<PREC, QH, INT>(geo, hA, phi_shift, xq, yq, zq, m, bt);
-    ring[slot][(ty + 1) * PW + tx + 1] = (PhiT)m[0];
-    if constexpr (F16) pring[slot][(ty + 1) * PW + tx + 1] = ld_pshift(pg_in, xq + geo.nx * (yq + geo.ny * zq));
+    const unsigned c = xq + geo.nx * (yq + geo.ny * zq);
+    CellOff o;
+    if (F16) o = off_xyz(geo, xq, yq, zq, SOLID ? __ldg(links + c) : 0u);
+    const Mom<V> m = h_moments<PREC, QH, V>(
+        [&](int cx, int cy, int cz) {
+          const unsigned i = (unsigned)lq_index<QH>(cx, cy, cz);
+          return V{raw<PREC>(hA[i * N + c])};
+        },
+        [&](int cx, int cy, int cz) { return V{(R)__ldg(phi_shift + writer(c, o, cx, cy, cz))}; });
+    ring[slot][i0] = (PhiT)m.s.v;
+    if constexpr (F16) pring[pslot][i0] = ld_pshift(pg_in, c);
+    V* hm = &hmom[mslot][tid];
+    hm[0] = m.s;
+    hm[NT] = m.x;
+    hm[2 * NT] = m.y;
+    hm[3 * NT] = m.z;
+    hm[4 * NT] = m.xx;
+    hm[5 * NT] = m.yy;
+    hm[6 * NT] = m.zz;
+    hm[7 * NT] = m.xy;
+    hm[8 * NT] = m.yz;
+    hm[9 * NT] = m.xz;
 #pragma unroll
-    for (int k = 0; k < 10; ++k) hmom[mslot][k * NT + tid] = m[k];
-    if (tid < NRING) {
-      const unsigned br = SOLID ? __ldg(links + rxq + geo.nx * (ryq + geo.ny * zq)) : 0u;
-      ring[slot][rj * PW + ri] = (PhiT)phi_at_xyz<PREC, QH, INT>(geo, hA, phi_shift, rxq, ryq, zq, br);
-      if constexpr (F16) pring[slot][rj * PW + ri] = ld_pshift(pg_in, rxq + geo.nx * (ryq + geo.ny * zq));
+    for (int r0 = 0; r0 < NRING; r0 += NT) {
+      const int r = r0 + tid;
+      if (r < NRING) {
+        int ri, rj;
+        frame_pos(r, PW, PH, ri, rj);
+        const unsigned rx = (unsigned)wrap_or_clamp(x0 - 1 + ri, (int)geo.nx, geo.wall[0]);
+        const unsigned ry = (unsigned)wrap_or_clamp(y0 - 1 + rj, (int)geo.ny, geo.wall[1]);
+        ring[slot][rj * PW + ri] = phi_at(rx, ry, zq);
+        if constexpr (F16) pring[pslot][rj * PW + ri] = ld_pshift(pg_in, rx + geo.nx * (ry + geo.ny * zq));
+      }
     }
   };
+  // in-plane part of the stencil of the plane in a ring slot
+  auto plane = [&](int slot) {
+    return phi_plane<V>([&](int cx, int cy) { return V{(R)ring[slot][i0 + cy * PW + cx]}; });
+  };
 
+  // g moments of the own cell of plane z (plane count b)
+  unsigned cell = 0;
+  CellOff o;
+  Mom<V> gm;
+  auto gather_g = [&](int b) {
+    gm = g_moments<PREC, QG, V>(
+        [&](int cx, int cy, int cz) {
+          const unsigned i = (unsigned)lq_index<QG>(cx, cy, cz);
+          return V{raw<PREC>(gA[i * N + cell])};
+        },
+        [&](int cx, int cy, int cz) {  // p* of the writer x - c, or of the cell itself after a bounce-back
+          const float* p0 = pring[FLAT ? 0 : b % NSP];
+          const float* pz = FLAT ? p0 : pring[(b - cz) % NSP];
+          return V{o.valid(-cx, -cy, -cz) ? (R)pz[i0 - cy * PW - cx] : (R)p0[i0]};
+        });
+  };
+
+  // Planes z0 - 1 .. z1 are filled in turn; once plane z + 1 is, plane z
+  // collides (a single plane: filled and collided at once).
+  PhiPlane<V> pm = {}, po = {}, pp = {};
   prefetch_plane(z0);
-  if (FLAT) {
-    fill(0, 0, 0);
-  } else {
-    fill(z0 - 1, 0, 1);  // moments of plane z0 - 1 are never used (written to the spare slot)
-    fill(z0, 1, 0);
-  }
-  for (int z = z0; z < z1; ++z) {
-    const int b = z - (z0 - 1);
-    if (!FLAT) fill(z + 1, (b + 1) % NS, (z + 1 - z0) & 1);
+  for (int zp = FLAT ? z0 : z0 - 1; zp <= (FLAT ? z0 : z1); ++zp) {
+    const int z = FLAT ? zp : zp - 1;
+    const int bp = zp - (z0 - 1), b = bp - 1;  // plane counts from z0 - 1
+    fill(FLAT ? 0 : zp, FLAT ? 0 : bp % NS, FLAT ? 0 : bp % NSP, FLAT ? 0 : bp & 1);
     __syncthreads();
-    if (!FLAT) prefetch_plane(z + 1);
-    const unsigned cell = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)z);
+    if (!FLAT && z >= z0) prefetch_plane(z + 1);
+    if (MARCH) (FLAT ? po : pp) = plane(FLAT ? 0 : bp % NS);
+    if (!FLAT && z < z0) {
+      pm = po;
+      po = pp;
+      continue;
+    }
+    cell = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)z);
     const unsigned blk = (SOLID && active) ? __ldg(links + cell) : 0u;
+    o = off_xyz(geo, (unsigned)x, (unsigned)y, (unsigned)z, blk);
     if (SOLID && active && (blk & SOLID_SELF)) {
       phi_out[cell] = (PhiT)0;  // solid cells are not updated; their populations stay zero
     } else if (active) {
-      const typename OffOf<INT>::T o = OffOf<INT>::at(geo, (unsigned)x, (unsigned)y, (unsigned)z, blk);
-      SmemPhi<PREC, FLAT, PW> at;
-      if (FLAT) {
-        at.plane[0] = at.plane[1] = at.plane[2] = ring[0];
+      const PhiT* at0 = ring[FLAT ? 0 : b % NS];
+      phi_out[cell] = at0[i0];
+      gather_g(b);
+      CellOut<PREC, QH, 1> out{hB, gB, N, cell, o, pg_out, Dither{F16 ? hash32(cell * 0x9E3779B1u + seed) : 0u}};
+      const V* hp = &hmom[FLAT ? 0 : b & 1][tid];
+      auto hm = [&] {
+        return Mom<V>{hp[0], hp[NT], hp[2 * NT], hp[3 * NT], hp[4 * NT], hp[5 * NT], hp[6 * NT], hp[7 * NT], hp[8 * NT], hp[9 * NT]};
+      };
+      // phi around the cell; a solid neighbour reads as the cell itself (neutral wetting)
+      auto at = [&](int cx, int cy, int cz) {
+        if (blk & link_bit(cx, cy, cz)) return (R)at0[i0];
+        return (R)(FLAT ? at0 : ring[(b + cz) % NS])[i0 + cy * PW + cx];
+      };
+      if constexpr (PREC == 1) {
+        collide_pairs<QH>(ph, at, gm, hm, out);
+      } else if constexpr (MARCH) {
+        collide<PREC, QH, V>(ph, po.c, FLAT ? phi_grad_flat(po) : phi_grad(pm, po, pp), gm, hm, out);
       } else {
-        at.plane[0] = ring[(b - 1) % NS];
-        at.plane[1] = ring[b % NS];
-        at.plane[2] = ring[(b + 1) % NS];
+        auto splane = [&](int cz) { return phi_plane<V>([&](int cx, int cy) { return V{at(cx, cy, cz)}; }); };
+        const PhiPlane<V> p0 = splane(0);
+        collide<PREC, QH, V>(ph, p0.c, QG == 9 ? phi_grad_flat(p0) : phi_grad(splane(-1), p0, splane(1)), gm, hm, out);
       }
-      // with one z plane the z neighbours are the plane itself (periodic or mirrored)
-      at.i0 = (ty + 1) * PW + (tx + 1);
-      at.blk = blk;
-      SmemShift<FLAT, PW> psh;
-      if constexpr (F16) {
-        if (FLAT) {
-          psh.plane[0] = psh.plane[1] = psh.plane[2] = pring[0];
-        } else {
-          psh.plane[0] = pring[(b - 1) % NS];
-          psh.plane[1] = pring[b % NS];
-          psh.plane[2] = pring[(b + 1) % NS];
-        }
-        psh.i0 = at.i0;
-      }
-      phi_out[cell] = (PhiT)at(0, 0, 0);
-      collide_cell<PREC, QH, 0, 1, SmemPhi<PREC, FLAT, PW>, 1, SmemShift<FLAT, PW>, typename OffOf<INT>::T>(
-          geo, ph, o, hA, gA, hB, gB, at, phi_shift, cell, seed, &hmom[FLAT ? 0 : ((z - z0) & 1)][tid], NT, psh,
-          pg_out);
+    }
+    if (!FLAT) {
+      pm = po;
+      po = pp;
     }
     if (NS == 3) __syncthreads();
   }
-  };
-  const bool interior = !SOLID && PFL_ZM_INTERIOR && x0 >= 2 && x0 + TX + 1 < (int)geo.nx && y0 >= 2 &&
-                        y0 + TY + 1 < (int)geo.ny && (FLAT || (z0 >= 2 && z1 + 1 < (int)geo.nz));
-  if (interior)
-    march(std::integral_constant<int, 1>());
-  else
-    march(std::integral_constant<int, 0>());
 }
 
+// grid: (ceil(nx / ZM_TX), ceil(ny / TY), ceil(nz / zc)), block ZM_TX x TY with
+// TY = zm_ty(FLAT).
+// tclock (launches replayed from a CUDA graph): the FP16 rounding seed comes
+// from the step count *tclock + tofs in device memory instead of `seed`, the
+// same function of the step count as the host's.
 template <int PREC, int QH, int FLAT, int SOLID = 0>
-__global__ void __launch_bounds__(ZM_TX * zm_ty(FLAT), (PREC == 0 ? PFL_ZM_MINB_FP64 : PFL_ZM_MINB) * ZM_TY / zm_ty(FLAT))
-    k_step_zm(Geo32 geo, Phys ph, const typename Store<PREC>::S* __restrict__ hA,
+__global__ void __launch_bounds__(ZM_TX* zm_ty(FLAT), zm_minb(PREC, ZM_TX* zm_ty(FLAT)))
+    k_step_zm(Geo32 geo, typename StepV<PREC>::Par ph, const typename Store<PREC>::S* __restrict__ hA,
               const typename Store<PREC>::S* __restrict__ gA, typename Store<PREC>::S* __restrict__ hB,
               typename Store<PREC>::S* __restrict__ gB, const typename Store<PREC>::PhiT* __restrict__ phi_shift,
               typename Store<PREC>::PhiT* __restrict__ phi_out, int zc, unsigned seed,
