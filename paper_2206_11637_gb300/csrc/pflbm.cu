@@ -113,6 +113,7 @@ struct pfl_ctx {
   int ab;        // two-array step: 0 = first pair current, 1 = second
   bool stale;    // two-array step: phi of the current state not yet materialised
   int zc;        // two-array step: z planes per block
+  int zc_push;   // the same of the 32 x 8 tiles without tensor copies (the adjoint's)
   long long t;   // steps taken
   int swapped;   // 1 after an even step (populations await the gather read)
   int qh;        // phase-field lattice: 15, 27 or 9 velocities
@@ -126,9 +127,22 @@ struct pfl_ctx {
   bool capturing;           // launches are being captured: pass the clock
   long long cap_t0;         // step count when the capture began
   long long clock_t;        // step count the device clock holds (-1: unknown)
+  // fused step with its loads by tensor copies: tile shape (index into
+  // TMA_TILES, -1: not used), maps of the two array pairs, and the host word a
+  // kernel reports to when a copy did not arrive
+  int tma;
+  StepMaps maps[2];
+  int* err;
+  bool wide;     // fused step without copies in tiles of WIDE_TX x WIDE_TY
 };
 
 namespace {
+
+pfl_status check_err(const pfl_ctx* c) {
+  if (c->err && *(volatile int*)c->err)
+    return fail(PFL_ERR_CUDA, "a copy of the fused step did not arrive; the state is not valid");
+  return PFL_OK;
+}
 
 // current populations (the two-array step alternates between two pairs)
 template <int PREC>
@@ -198,6 +212,143 @@ void launch_phi(pfl_ctx* c) {
   c->cur = 1 - c->cur;
 }
 
+// z planes per block of the fused step in tiles of tx x ty, at most `most`.
+// Every block marches zc planes and fills two more (the planes below and above
+// its first) before it starts, about half a plane's work; blocks run in waves
+// of `slots` resident blocks.  The zc with the least modelled time:
+// waves x (zc + 0.5).
+int z_chunk(const pfl_params* p, int tx, int ty, long long slots, int most) {
+  const long long bxy = (long long)((p->nx + tx - 1) / tx) * ((p->ny + ty - 1) / ty);
+  int best = std::min(p->nz, most);
+  double best_cost = 1e300;
+  for (int zc = best; zc >= 1; --zc) {
+    const long long blocks = bxy * ((p->nz + zc - 1) / zc);
+    const double cost = (double)((blocks + slots - 1) / slots) * (zc + 0.5);
+    if (cost < best_cost * (1 - 1e-9)) {
+      best_cost = cost;
+      best = zc;
+    }
+  }
+  return best;
+}
+
+// share of the threads of tx x ty tiles that hold a cell
+double tile_use(const pfl_params* p, int tx, int ty) {
+  auto part = [](int n, int t) { return (double)n / ((n + t - 1) / t * t); };
+  return part(p->nx, tx) * part(p->ny, ty);
+}
+
+// Tiles of 64 x 4 for the FP32 step without copies (rows that are no whole
+// 16-byte units, solid cells): longer runs of each stream, for more ring phi.
+// GLUPS of 64 x 4 and 32 x 8: bubble 186x378x153 13.9 and 12.7 (D3Q27 10.8 and
+// 10.2), drop 98^3 11.8 and 10.4, Taylor tube 98x960x98 11.1 and 10.8; where
+// more lanes idle, drop 130^3 10.8 and 11.7, tube 66x640x66 9.3 and 9.7; and no
+// gain at the size of L2, bubble 61x183x61 11.7 and 11.8.
+constexpr int WIDE_TX = 64, WIDE_TY = 4;
+bool wide_tile(const pfl_params* p) {
+  return uses_two_arrays(p) && p->precision == PFL_FP32 && p->nz > 1 && qh_of(p) != 9 &&
+         (long long)p->nx * p->ny * p->nz >= 900000 && tile_use(p, WIDE_TX, WIDE_TY) >= 0.95 * tile_use(p, ZM_TX, ZM_TY);
+}
+
+// Tiles of the fused step by tensor copies (wide rows and z chunks of at most
+// TMA_ZC planes).  What a step moves is 84 streams, and how much of the HBM rate
+// they get depends on how long a run of each is touched at a time: copying them
+// with no arithmetic, tiles of 32 x 8 marching 64 planes reach 4.4 TB/s, 8 planes
+// 5.3, 128 x 2 and 8 planes 5.9, whole planes in order 6.8.  Wide tiles repeat
+// more ring phi (264 of 256 cells), which the copies hide: 128x384x128 bubble,
+// FP32, GLUPS at 12 planes: 128 x 2 17.0, 128 x 3 16.5, 64 x 4 16.1, 32 x 8 14.6,
+// and 14.6 for 32 x 8 without the copies; 128 x 2 at 6, 20 and 32 planes 16.7,
+// 17.0 and 16.2.
+constexpr int NTMA = 2;
+constexpr int TMA_TILES[NTMA][2] = {{128, 2}, {64, 4}};
+constexpr int TMA_ZC = 12;
+constexpr long long TMA_CELLS = 1 << 19;
+
+typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// The kernel of a tile, its dynamic shared memory and, on request, its launch.
+template <int PREC, int QH, int J>
+struct TmaStep {
+  static constexpr int TX = TMA_TILES[J][0], TY = TMA_TILES[J][1];
+  static constexpr int BYTES = (QH + qg_of<QH>()) * TX * TY * (int)sizeof(typename Store<PREC>::S);
+  static bool prepare(int* per_sm) {
+    return cudaFuncSetAttribute(k_step_tma<PREC, QH, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, BYTES) == cudaSuccess &&
+           cudaFuncSetAttribute(k_step_tma<PREC, QH, TX, TY>, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess &&
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_step_tma<PREC, QH, TX, TY>, TX * TY, BYTES) == cudaSuccess;
+  }
+  template <class... A>
+  static void launch(const pfl_ctx* c, cudaLaunchConfig_t cfg, A... args) {
+    cfg.gridDim = dim3((c->p.nx + TX - 1) / TX, (c->p.ny + TY - 1) / TY, (c->p.nz + c->zc - 1) / c->zc);
+    cfg.blockDim = dim3(TX, TY);
+    cfg.dynamicSmemBytes = BYTES;
+    cudaLaunchKernelEx(&cfg, k_step_tma<PREC, QH, TX, TY>, args...);
+  }
+};
+// fn(TmaStep<PREC, QH, j>()) of the shape index j
+template <int PREC, int QH, class F>
+void tma_shape(int j, const F& fn) {
+  if (j == 0) fn(TmaStep<PREC, QH, 0>());
+  if (j == 1) fn(TmaStep<PREC, QH, 1>());
+}
+template <int PREC, int QH>
+constexpr bool has_tma() {
+  return PREC == 1 && QH != 9;
+}
+
+// The tile a lattice takes (-1: 32 x 8 without copies).  Copies need rows of
+// whole 16-byte units (tensor-map strides), no solid cells, and pay on FP32
+// lattices beyond L2 (GLUPS with and without: 128x96x48 13.4 and 12.2, 64^3 10.1
+// and 11.1; FP16S is bound by instruction issue, 15.2 and 15.7).  Among the
+// tiles, the best use of the lanes times the tile's own rate (128 x 2 : 64 x 4 :
+// 32 x 8 as 1 : 0.95 : 0.85; idle lanes cost the narrow tile less).  Measured,
+// 128 x 2, 64 x 4, 32 x 8: 100 wide 12.4, 12.0, 10.9; 144 wide 10.3, 12.8, 13.8;
+// 192 wide 13.5, 14.9, 13.5; 200 wide 14.4, 13.6, 13.1.
+int tma_tile(const pfl_params* p) {
+  if (!uses_two_arrays(p) || p->precision != PFL_FP32 || p->solids || p->nz < 2 || qh_of(p) == 9) return -1;
+  if (p->nx % 4 != 0 || (long long)p->nx * p->ny * p->nz < TMA_CELLS) return -1;
+  const double rate[NTMA] = {1.0, 0.95};
+  int best = -1;
+  double most = 0.85 * tile_use(p, ZM_TX, ZM_TY);
+  for (int j = 0; j < NTMA; ++j) {
+    const double r = rate[j] * tile_use(p, TMA_TILES[j][0], TMA_TILES[j][1]);
+    if (r > most) {
+      most = r;
+      best = j;
+    }
+  }
+  return best;
+}
+
+// Tensor maps of the two array pairs, launch attributes, the error word and the
+// z chunk of a context that takes tile shape c->tma.
+template <int PREC, int QH>
+void setup_tma_t(pfl_ctx* c, EncodeTiled enc, int sms, bool* ok) {
+  if constexpr (has_tma<PREC, QH>()) {
+    const int tx = TMA_TILES[c->tma][0], ty = TMA_TILES[c->tma][1];
+    const cuuint64_t S = sizeof(typename Store<PREC>::S), nx = c->p.nx, ny = c->p.ny, nz = c->p.nz, N = nx * ny * nz;
+    auto make = [&](CUtensorMap* m, size_t off, cuuint32_t q) {
+      const cuuint64_t dims[4] = {nx, ny, nz, q}, strides[3] = {nx * S, nx * ny * S, N * S};
+      const cuuint32_t box[4] = {(cuuint32_t)tx, (cuuint32_t)ty, 1, q}, es[4] = {1, 1, 1, 1};
+      return enc(m, PREC == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, c->ws + off, dims, strides,
+                 box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    *ok = make(&c->maps[0].h, c->L.h, QH) && make(&c->maps[0].g, c->L.g, 27) && make(&c->maps[1].h, c->L.h2, QH) &&
+          make(&c->maps[1].g, c->L.g2, 27);
+    int per_sm = 1;
+    tma_shape<PREC, QH>(c->tma, [&](auto k) { *ok = *ok && k.prepare(&per_sm); });
+    *ok = *ok && per_sm > 0 && cudaHostAlloc((void**)&c->err, 64, cudaHostAllocPortable) == cudaSuccess;
+    if (!*ok) return;
+    *c->err = 0;
+    const long long slots = (long long)sms * per_sm;
+    const long long blocks = (long long)((c->p.nx + tx - 1) / tx) * ((c->p.ny + ty - 1) / ty) * ((c->p.nz + TMA_ZC - 1) / TMA_ZC);
+    // from two waves on the last one's share is small and the march's length counts
+    c->zc = blocks >= 2 * slots ? TMA_ZC : z_chunk(&c->p, tx, ty, slots, TMA_ZC);
+  }
+}
+
 // One collide-stream launch (without the phi pass that completes an in-place
 // step).  Two-array contexts run the fused kernel; MRT in place the pair-based
 // kernel; the BGK test mode, and lattices too large for 32-bit indices, the
@@ -225,15 +376,30 @@ void step_only(pfl_ctx* c) {
     const typename Store<PREC>::PhiT* shift = phishift<PREC>(c);
     const unsigned long long* tclock = c->capturing ? clock_of(c) : nullptr;
     const int tofs = (int)(c->t - c->cap_t0);
-#define PFL_ZM(FLAT, SOLID)                                                                                   \
-  cudaLaunchKernelEx(&cfg, k_step_zm<PREC, QH, FLAT, SOLID>, c->g32, ph1, ha, ga, hnext<PREC>(c),            \
-                     gnext<PREC>(c), shift, phicur<PREC>(c), c->zc, step_seed(c), links, tclock, tofs,       \
+    if (c->tma >= 0) {
+      if constexpr (has_tma<PREC, QH>())
+        tma_shape<PREC, QH>(c->tma, [&](auto k) {
+          k.launch(c, cfg, c->maps[c->ab], c->g32, ph1, ha, ga, hnext<PREC>(c), gnext<PREC>(c), shift, phicur<PREC>(c), c->zc,
+                   step_seed(c), tclock, tofs, (const __half*)pgshift(c), pgcur(c), (volatile int*)c->err);
+        });
+    } else
+#define PFL_ZM(...)                                                                                      \
+  cudaLaunchKernelEx(&cfg, k_step_zm<PREC, QH, __VA_ARGS__>, c->g32, ph1, ha, ga, hnext<PREC>(c),       \
+                     gnext<PREC>(c), shift, phicur<PREC>(c), c->zc, step_seed(c), links, tclock, tofs,  \
                      (const __half*)pgshift(c), pgcur(c))
     if (c->p.nz == 1) {
       if (c->solid)
         PFL_ZM(1, 1);
       else
         PFL_ZM(1, 0);
+    } else if (PREC == 1 && QH != 9 && c->wide) {
+      constexpr int P = PREC == 1 && QH != 9 ? WIDE_TX : ZM_TX, Q = PREC == 1 && QH != 9 ? WIDE_TY : ZM_TY;
+      cfg.gridDim = dim3((c->p.nx + P - 1) / P, (c->p.ny + Q - 1) / Q, (c->p.nz + c->zc - 1) / c->zc);
+      cfg.blockDim = dim3(P, Q);
+      if (c->solid)
+        PFL_ZM(0, 1, P, Q);
+      else
+        PFL_ZM(0, 0, P, Q);
     } else {
       if (c->solid)
         PFL_ZM(0, 1);
@@ -425,6 +591,23 @@ void launch_umax(pfl_ctx* c, double* part, double* out) {
     }                                                                         \
   } while (0)
 
+bool setup_tma(pfl_ctx* c, int sms) {
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess)
+    return false;
+  bool ok = true;
+  DISPATCH(c, setup_tma_t, c, (EncodeTiled)fn, sms, &ok);
+  return ok;
+}
+
+// Releases what the context holds on the host.
+void free_ctx(pfl_ctx* c) {
+  if (c->err) cudaFreeHost(c->err);
+  delete c;
+}
+
 // Copy n doubles from a host or device source into the device at dst.
 pfl_status to_device(pfl_ctx* c, double* dst, const double* src, size_t n) {
   CUDA_TRY(cudaMemcpyAsync(dst, src, n * sizeof(double), cudaMemcpyDefault, c->stream));
@@ -603,34 +786,24 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
   c->capturing = false;
   c->cap_t0 = 0;
   c->clock_t = -1;
+  c->err = nullptr;
   {
-    // z planes per block.  Every block marches zc planes and fills two more
-    // (the planes below and above its first) before it starts, about half a
-    // plane's work; blocks run in waves of `slots` resident blocks.  Take the
-    // zc with the least modelled time: waves x (zc + 0.5).
     int sms = 152, per_sm = 2;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    const dim3 blk(ZM_TX, ZM_TY);
     if (p->precision == PFL_FP64)
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_zm<0, 15, 0>, (int)(blk.x * blk.y), 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_zm<0, 15, 0>, ZM_TX * ZM_TY, 0);
     else if (p->precision == PFL_FP32)
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_zm<1, 15, 0>, (int)(blk.x * blk.y), 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_zm<1, 15, 0>, ZM_TX * ZM_TY, 0);
     else
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_zm<2, 15, 0>, (int)(blk.x * blk.y), 0);
-    if (per_sm < 1) per_sm = 1;
-    const long long slots = (long long)sms * per_sm;
-    const long long bxy = (long long)((p->nx + ZM_TX - 1) / ZM_TX) * ((p->ny + ZM_TY - 1) / ZM_TY);
-    int best = p->nz;
-    double best_cost = 1e300;
-    for (int zc = p->nz; zc >= 1; --zc) {
-      const long long blocks = bxy * ((p->nz + zc - 1) / zc);
-      const double cost = (double)((blocks + slots - 1) / slots) * (zc + 0.5);
-      if (cost < best_cost * (1 - 1e-9)) {
-        best_cost = cost;
-        best = zc;
-      }
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_zm<2, 15, 0>, ZM_TX * ZM_TY, 0);
+    c->zc_push = c->zc = z_chunk(p, ZM_TX, ZM_TY, (long long)sms * (per_sm < 1 ? 1 : per_sm), p->nz);
+    c->tma = tma_tile(p);
+    c->wide = c->tma < 0 && wide_tile(p);
+    if (c->wide) c->zc = z_chunk(p, WIDE_TX, WIDE_TY, (long long)sms * PFL_ZM_MINB, p->nz);
+    if (c->tma >= 0 && !setup_tma(c, sms)) {
+      free_ctx(c);
+      return fail(PFL_ERR_CUDA, "setting up the tensor maps of the fused step");
     }
-    c->zc = best;
   }
   c->geo.nx = p->nx;
   c->geo.ny = p->ny;
@@ -647,7 +820,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
   for (int a = 0; a < 3; ++a) c->g32.wall[a] = c->geo.wall[a];
   if (c->idx32 && (!fastdiv_ok((unsigned)p->nx, (unsigned)c->geo.N) ||
                    !fastdiv_ok((unsigned)p->ny, (unsigned)(c->geo.N / p->nx)))) {
-    delete c;
+    free_ctx(c);
     return fail(PFL_ERR_STATE, "integer divider self-check failed");
   }
   c->ph.rho_h = p->rho_h;
@@ -672,7 +845,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
       phi_host.resize((size_t)N);
       cudaError_t e = cudaMemcpy(phi_host.data(), phi0, (size_t)N * sizeof(double), cudaMemcpyDeviceToHost);
       if (e != cudaSuccess) {
-        delete c;
+        free_ctx(c);
         return cuda_fail(e, "phi0 to the host for the hydrostatic start");
       }
       ph0 = phi_host.data();
@@ -697,19 +870,19 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
       double* a_p = st + 4 * cnt;
       pfl_status s;
       if ((s = to_device(c, a_phi, phi0 + c0, cnt)) != PFL_OK) {
-        delete c;
+        free_ctx(c);
         return s;
       }
       if (u0 && pass == 1) {
         if ((s = to_device(c, a_ux, u0 + c0, cnt)) != PFL_OK || (s = to_device(c, a_uy, u0 + N + c0, cnt)) != PFL_OK ||
             (s = to_device(c, a_uz, u0 + 2 * N + c0, cnt)) != PFL_OK) {
-          delete c;
+          free_ctx(c);
           return s;
         }
       }
       if (p0) {
         if ((s = to_device(c, a_p, p0 + c0, cnt)) != PFL_OK) {
-          delete c;
+          free_ctx(c);
           return s;
         }
       }
@@ -723,7 +896,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
       cudaError_t e = cudaStreamSynchronize(c->stream);
       if (e == cudaSuccess) e = cudaGetLastError();
       if (e != cudaSuccess) {
-        delete c;
+        free_ctx(c);
         return cuda_fail(e, "initialisation");
       }
     }
@@ -731,7 +904,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
   DISPATCH_S(s, c, fresh_phi, c, false);
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (s != PFL_OK || e != cudaSuccess) {
-    delete c;
+    free_ctx(c);
     return s != PFL_OK ? s : cuda_fail(e, "initial phi");
   }
   *out = c;
@@ -744,6 +917,7 @@ pfl_status pfl_step(pfl_ctx* c, int n) {
   CUDA_TRY(on_device.enter(c->device));
   if (n < 0) return fail(PFL_ERR_ARG, "n_steps must be >= 0");
   if (n == 0) return PFL_OK;
+  if (pfl_status e = check_err(c)) return e;
   if (c->zm && c->graph_k > 0 && n >= c->graph_k) {
     // whole graphs of graph_k steps, unless the caller is capturing the stream
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -800,7 +974,7 @@ pfl_status pfl_fields(pfl_ctx* c, double* phi, double* rho, double* p, double* u
   }
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return PFL_OK;
+  return check_err(c);
 }
 
 pfl_status pfl_populations(pfl_ctx* c, double* h, double* g) {
@@ -825,7 +999,7 @@ pfl_status pfl_populations(pfl_ctx* c, double* h, double* g) {
     }
   }
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return PFL_OK;
+  return check_err(c);
 }
 
 pfl_status pfl_set_populations(pfl_ctx* c, const double* h, const double* g) {
@@ -934,7 +1108,7 @@ pfl_status pfl_save(pfl_ctx* c, void* buf, size_t bytes) {
     off += hd.bytes[k];
   }
   CUDA_TRY(cudaStreamSynchronize(c->stream));  // the header lives on this stack
-  return PFL_OK;
+  return check_err(c);
 }
 
 pfl_status pfl_load(pfl_ctx* c, const void* buf, size_t bytes) {
@@ -1034,7 +1208,7 @@ pfl_status pfl_diag(pfl_ctx* c, double out[8], long long* nonfinite) {
   if (!(umax <= PFL_SPEED_LIMIT))
     return fail(PFL_ERR_UNSTABLE, "flow speed |u| = " + std::to_string(umax) + " exceeds " +
                                       std::to_string(PFL_SPEED_LIMIT) + " (lattice units)");
-  return PFL_OK;
+  return check_err(c);
 }
 
 pfl_status pfl_max_speed(pfl_ctx* c, double* umax) {
@@ -1047,7 +1221,7 @@ pfl_status pfl_max_speed(pfl_ctx* c, double* umax) {
   if (st != PFL_OK) return st;
   CUDA_TRY(cudaMemcpyAsync(umax, ures, sizeof(double), cudaMemcpyDefault, c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return PFL_OK;
+  return check_err(c);
 }
 
 pfl_status pfl_interface_height(pfl_ctx* c, int x, int z, double* y) {
@@ -1062,7 +1236,7 @@ pfl_status pfl_interface_height(pfl_ctx* c, int x, int z, double* y) {
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaMemcpyAsync(y, res, sizeof(double), cudaMemcpyDefault, c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return PFL_OK;
+  return check_err(c);
 }
 
 pfl_status pfl_kernel_times(pfl_ctx* c, int n, double ms[2]) {
@@ -1203,8 +1377,8 @@ void launch_adj_step(pfl_ctx* c, const AdjLayout& A, char* aws, char* slot, int 
   else
     k_adj_local<PREC, QH, 0><<<nb, ADJ_THREADS, 0, c->stream>>>(c->g32, phr, ap, h, g, phi, (const R*)lam_in,
                                                              acc, (R*)lam_out, aux, part);
-  const dim3 grid((c->p.nx + ZM_TX - 1) / ZM_TX, (c->p.ny + ZM_TY - 1) / ZM_TY, (c->p.nz + c->zc - 1) / c->zc);
-  k_adj_phi<R, qg_of<QH>()><<<grid, dim3(ZM_TX, ZM_TY), 0, c->stream>>>(c->g32, aux, acc, W, c->zc);
+  const dim3 grid((c->p.nx + ZM_TX - 1) / ZM_TX, (c->p.ny + ZM_TY - 1) / ZM_TY, (c->p.nz + c->zc_push - 1) / c->zc_push);
+  k_adj_phi<R, qg_of<QH>()><<<grid, dim3(ZM_TX, ZM_TY), 0, c->stream>>>(c->g32, aux, acc, W, c->zc_push);
 }
 
 // lambda at the final time: local part 0, acc = W (the objective's weight on
@@ -1237,13 +1411,13 @@ struct SlotPtr {
 template <int PREC, int QH>
 void zm_step_slots(pfl_ctx* c, const SlotPtr<PREC>& a, const SlotPtr<PREC>& b) {
   const int ty = zm_ty(c->p.nz == 1);
-  const dim3 grid((c->p.nx + ZM_TX - 1) / ZM_TX, (c->p.ny + ty - 1) / ty, (c->p.nz + c->zc - 1) / c->zc);
+  const dim3 grid((c->p.nx + ZM_TX - 1) / ZM_TX, (c->p.ny + ty - 1) / ty, (c->p.nz + c->zc_push - 1) / c->zc_push);
   const dim3 block(ZM_TX, ty);
   const typename StepV<PREC>::Par ph = step_par<PREC>(c->ph);
   if (c->p.nz == 1)
-    k_step_zm<PREC, QH, 1><<<grid, block, 0, c->stream>>>(c->g32, ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc, 0u);
+    k_step_zm<PREC, QH, 1><<<grid, block, 0, c->stream>>>(c->g32, ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc_push, 0u);
   else
-    k_step_zm<PREC, QH, 0><<<grid, block, 0, c->stream>>>(c->g32, ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc, 0u);
+    k_step_zm<PREC, QH, 0><<<grid, block, 0, c->stream>>>(c->g32, ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc_push, 0u);
 }
 
 // Adjoint with the fused two-array engine.  Forward sweep: checkpoints every K
@@ -1474,7 +1648,7 @@ void pfl_destroy(pfl_ctx* c) {
   cudaStreamSynchronize(c->stream);
   drop_graphs(c);
   if (c->cap) cudaStreamDestroy(c->cap);
-  delete c;
+  free_ctx(c);
 }
 
 }  // extern "C"

@@ -23,6 +23,7 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "tma.cuh"
 #include "vec.cuh"
 
 #ifndef PFL_STEP_THREADS
@@ -801,10 +802,12 @@ __device__ __forceinline__ void collide_pairs(const PhysR<float>& par, const Phi
     const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
     const V a{phi_at(cx, cy, cz)}, b{phi_at(-cx, -cy, -cz)};
     const V w = vbc<V>(lq_w<QG>(i)), d = a - b;
-    if (cx) gx = vfma(cx > 0 ? w : -w, d, gx);
-    if (cy) gy = vfma(cy > 0 ? w : -w, d, gy);
-    if (cz) gz = vfma(cz > 0 ? w : -w, d, gz);
-    lap = vfma(w, (a - pc) + (b - pc), lap);  // differences first: exact for nearby values
+    const V t = (a - pc) + (b - pc);  // differences first: exact for nearby values
+    // (member 0 has every component of the lattice)
+    if (cx) gx = i ? vfma(cx > 0 ? w : -w, d, gx) : (cx > 0 ? w : -w) * d;
+    if (cy) gy = i ? vfma(cy > 0 ? w : -w, d, gy) : (cy > 0 ? w : -w) * d;
+    if (cz) gz = i ? vfma(cz > 0 ? w : -w, d, gz) : (cz > 0 ? w : -w) * d;
+    lap = i ? vfma(w, t, lap) : w * t;
   }
   gx = gx * three;
   gy = gy * three;
@@ -855,16 +858,15 @@ __device__ __forceinline__ void collide_pairs(const PhysR<float>& par, const Phi
 #pragma unroll
     for (int i = 0; i < GR; ++i) {
       const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
-      V E = zero, L = zero;
-      if (cx) E = E + Gxx;
-      if (cy) E = E + Gyy;
-      if (cz) E = E + Gzz;
+      V E = cx ? Gxx : (cy ? Gyy : Gzz);
+      if (cx && cy) E = E + Gyy;
+      if ((cx || cy) && cz) E = E + Gzz;
       if (cx && cy) E = E + ((cx * cy > 0) ? Gxy : -Gxy);
       if (cy && cz) E = E + ((cy * cz > 0) ? Gyz : -Gyz);
       if (cx && cz) E = E + ((cx * cz > 0) ? Gxz : -Gxz);
-      if (cx) L = L + (cx > 0 ? bx : -bx);
-      if (cy) L = L + (cy > 0 ? by : -by);
-      if (cz) L = L + (cz > 0 ? bz : -bz);
+      V L = cx ? (cx > 0 ? bx : -bx) : (cy ? (cy > 0 ? by : -by) : (cz > 0 ? bz : -bz));
+      if (cx && cy) L = L + (cy > 0 ? by : -by);
+      if ((cx || cy) && cz) L = L + (cz > 0 ? bz : -bz);
       out.g_(i, QG - 1 - i, cx, cy, cz, wsum(lq_w<QG>(i), pst, als + (E + L)), wsum(lq_w<QG>(i), pst, als + (E - L)));
     }
   }
@@ -887,20 +889,20 @@ __device__ __forceinline__ void collide_pairs(const PhysR<float>& par, const Phi
     const V by = vfma(tn, gy, vfma(p3, uy, a1 * vfma(-phl, uy, h.y)));
     const V bz = vfma(tn, gz, vfma(p3, uz, a1 * vfma(-phl, uz, h.z)));
     const V a22 = vbc<V>(2.0) * a2;
+    const V Hxx = a2 * dxx, Hyy = a2 * dyy, Hzz = a2 * dzz;
     out.hrest(wsum(hq_w<QH>(hq_rest<QH>()), phl, als));
 #pragma unroll
     for (int k = 0; k < hq_rest<QH>(); ++k) {
       const int cx = hq_cx<QH>(k), cy = hq_cy<QH>(k), cz = hq_cz<QH>(k);
-      V E = zero, L = zero;
-      if (cx) E = vfma(a2, dxx, E);
-      if (cy) E = vfma(a2, dyy, E);
-      if (cz) E = vfma(a2, dzz, E);
+      V E = cx ? Hxx : (cy ? Hyy : Hzz);
+      if (cx && cy) E = vfma(a2, dyy, E);
+      if ((cx || cy) && cz) E = vfma(a2, dzz, E);
       if (cx && cy) E = vfma((cx * cy > 0) ? a22 : -a22, h.xy, E);
       if (cy && cz) E = vfma((cy * cz > 0) ? a22 : -a22, h.yz, E);
       if (cx && cz) E = vfma((cx * cz > 0) ? a22 : -a22, h.xz, E);
-      if (cx) L = L + (cx > 0 ? bx : -bx);
-      if (cy) L = L + (cy > 0 ? by : -by);
-      if (cz) L = L + (cz > 0 ? bz : -bz);
+      V L = cx ? (cx > 0 ? bx : -bx) : (cy ? (cy > 0 ? by : -by) : (cz > 0 ? bz : -bz));
+      if (cx && cy) L = L + (cy > 0 ? by : -by);
+      if ((cx || cy) && cz) L = L + (cz > 0 ? bz : -bz);
       out.h_(k, QH - 1 - k, cx, cy, cz, wsum(hq_w<QH>(k), phl, als + (E + L)), wsum(hq_w<QH>(k), phl, als + (E - L)));
     }
   }
@@ -1108,15 +1110,20 @@ __device__ __forceinline__ CellOff off_xyz(const Geo32& geo, unsigned x, unsigne
 // batched engine's work list), run by a block of TX x TY threads.  The caller
 // has waited for the previous step.  SOLID: the lattice holds solid cells, given
 // by `links` (one word per cell).
-template <int PREC, int QH, int TY, int FLAT, int SOLID, int TX = ZM_TX>
-__device__ __forceinline__ void zm_tile(const Geo32& geo, const typename StepV<PREC>::Par& ph,
+// TM: the tile's own populations come by tensor copies into dynamic shared
+// memory, one box of every member of h and of g per plane, issued as soon as the
+// plane before is read; `mbar` holds the two barriers (h, g).  Returns false if
+// a copy did not arrive.
+template <int PREC, int QH, int TY, int FLAT, int SOLID, int TX = ZM_TX, int TM = 0>
+__device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<PREC>::Par& ph,
                                         const typename Store<PREC>::S* __restrict__ hA,
                                         const typename Store<PREC>::S* __restrict__ gA,
                                         typename Store<PREC>::S* __restrict__ hB, typename Store<PREC>::S* __restrict__ gB,
                                         const typename Store<PREC>::PhiT* __restrict__ phi_shift,
                                         typename Store<PREC>::PhiT* __restrict__ phi_out, int zc, unsigned seed,
                                         const unsigned* __restrict__ links, const __half* __restrict__ pg_in,
-                                        __half* __restrict__ pg_out, int bx, int by, int bz) {
+                                        __half* __restrict__ pg_out, int bx, int by, int bz,
+                                        const StepMaps* maps = nullptr, unsigned mbar = 0) {
   typedef typename Store<PREC>::PhiT PhiT;
   typedef typename Store<PREC>::S S;
   typedef typename Store<PREC>::R R;
@@ -1152,11 +1159,30 @@ __device__ __forceinline__ void zm_tile(const Geo32& geo, const typename StepV<P
 
   // L1 prefetch of the g populations plane zp's collision will read
   auto prefetch_plane = [&](int zp) {
-    if (!(PFL_ZM_PREFETCH && PREC == 1 && QH == 15 && !FLAT) || !active || zp >= z1) return;
+    if (!(PFL_ZM_PREFETCH && !TM && PREC == 1 && QH == 15 && !FLAT) || !active || zp >= z1) return;
     const unsigned c = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)zp);
 #pragma unroll
     for (int i = 0; i < QG; ++i) prefetch_l1(gA + (unsigned)i * N + c);
   };
+  // tensor copies: h of plane zp (wrapped or clamped), g of plane z
+  extern __shared__ __align__(128) unsigned char dyn[];
+  S* sG = (S*)dyn;
+  S* sH = sG + QG * NT;
+  unsigned phase_h = 0, phase_g = 0;
+  bool ok = true;
+  auto issue_h = [&](int zp) {
+    if (tid == 0) {
+      mbar_expect(mbar, QH * NT * sizeof(S));
+      tma4(smem_u32(sH), &maps->h, x0, y0, wrap_or_clamp(zp, (int)geo.nz, geo.wall[2]), 0, mbar);
+    }
+  };
+  auto issue_g = [&](int z) {
+    if (tid == 0) {
+      mbar_expect(mbar + 8, QG * NT * sizeof(S));
+      tma4(smem_u32(sG), &maps->g, x0, y0, z, 0, mbar + 8);
+    }
+  };
+
   // phi of cell (qx, qy, zq) from memory
   auto phi_at = [&](unsigned qx, unsigned qy, unsigned zq) {
     const unsigned c = qx + geo.nx * (qy + geo.ny * zq);
@@ -1170,13 +1196,16 @@ __device__ __forceinline__ void zm_tile(const Geo32& geo, const typename StepV<P
     const unsigned c = xq + geo.nx * (yq + geo.ny * zq);
     CellOff o;
     if (F16) o = off_xyz(geo, xq, yq, zq, SOLID ? __ldg(links + c) : 0u);
+    if constexpr (TM != 0) ok = mbar_wait(mbar, phase_h++ & 1) && ok;
     const Mom<V> m = h_moments<PREC, QH, V>(
         [&](int cx, int cy, int cz) {
           const unsigned i = (unsigned)lq_index<QH>(cx, cy, cz);
+          if constexpr (TM != 0) return V{raw<PREC>(sH[i * NT + tid])};
           return V{raw<PREC>(hA[i * N + c])};
         },
         [&](int cx, int cy, int cz) { return V{(R)__ldg(phi_shift + writer(c, o, cx, cy, cz))}; });
-    ring[slot][i0] = (PhiT)m.s.v;
+    // (tile positions outside the lattice serve as ring cells; the copy does not hold them)
+    ring[slot][i0] = TM && !active ? phi_at(xq, yq, zq) : (PhiT)m.s.v;
     if constexpr (F16) pring[pslot][i0] = ld_pshift(pg_in, c);
     V* hm = &hmom[mslot][tid];
     hm[0] = m.s;
@@ -1215,6 +1244,7 @@ __device__ __forceinline__ void zm_tile(const Geo32& geo, const typename StepV<P
     gm = g_moments<PREC, QG, V>(
         [&](int cx, int cy, int cz) {
           const unsigned i = (unsigned)lq_index<QG>(cx, cy, cz);
+          if constexpr (TM != 0) return V{raw<PREC>(sG[i * NT + tid])};
           return V{raw<PREC>(gA[i * N + cell])};
         },
         [&](int cx, int cy, int cz) {  // p* of the writer x - c, or of the cell itself after a bounce-back
@@ -1227,12 +1257,30 @@ __device__ __forceinline__ void zm_tile(const Geo32& geo, const typename StepV<P
   // Planes z0 - 1 .. z1 are filled in turn; once plane z + 1 is, plane z
   // collides (a single plane: filled and collided at once).
   PhiPlane<V> pm = {}, po = {}, pp = {};
+  if (TM) issue_h(z0 - 1);
   prefetch_plane(z0);
   for (int zp = FLAT ? z0 : z0 - 1; zp <= (FLAT ? z0 : z1); ++zp) {
     const int z = FLAT ? zp : zp - 1;
     const int bp = zp - (z0 - 1), b = bp - 1;  // plane counts from z0 - 1
+    // FP32 gathers g before the barrier, so that one barrier frees both copies;
+    // FP16S needs the p* shifts of plane z + 1 first
+    if (TM && !F16 && z >= z0) {
+      ok = mbar_wait(mbar + 8, phase_g++ & 1) && ok;
+      gather_g(b);
+    }
     fill(FLAT ? 0 : zp, FLAT ? 0 : bp % NS, FLAT ? 0 : bp % NSP, FLAT ? 0 : bp & 1);
-    __syncthreads();
+    if constexpr (TM != 0) {
+      if (!__syncthreads_and(ok)) {
+        // give the copies in flight another bounded wait before the block's memory goes
+        mbar_wait(mbar, phase_h & 1);
+        mbar_wait(mbar + 8, phase_g & 1);
+        return false;
+      }
+      if (zp < z1) issue_h(zp + 1);
+      if (zp < z1 && (F16 ? zp == z0 : zp >= z0)) issue_g(zp);
+    } else {
+      __syncthreads();
+    }
     if (!FLAT && z >= z0) prefetch_plane(z + 1);
     if (MARCH) (FLAT ? po : pp) = plane(FLAT ? 0 : bp % NS);
     if (!FLAT && z < z0) {
@@ -1243,12 +1291,18 @@ __device__ __forceinline__ void zm_tile(const Geo32& geo, const typename StepV<P
     cell = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)z);
     const unsigned blk = (SOLID && active) ? __ldg(links + cell) : 0u;
     o = off_xyz(geo, (unsigned)x, (unsigned)y, (unsigned)z, blk);
+    if (TM && F16) {
+      ok = mbar_wait(mbar + 8, phase_g++ & 1) && ok;
+      gather_g(b);
+      __syncthreads();
+      if (z + 1 < z1) issue_g(z + 1);
+    }
     if (SOLID && active && (blk & SOLID_SELF)) {
       phi_out[cell] = (PhiT)0;  // solid cells are not updated; their populations stay zero
     } else if (active) {
       const PhiT* at0 = ring[FLAT ? 0 : b % NS];
       phi_out[cell] = at0[i0];
-      gather_g(b);
+      if (!TM) gather_g(b);
       CellOut<PREC, QH, 1> out{hB, gB, N, cell, o, pg_out, Dither{F16 ? hash32(cell * 0x9E3779B1u + seed) : 0u}};
       const V* hp = &hmom[FLAT ? 0 : b & 1][tid];
       auto hm = [&] {
@@ -1275,15 +1329,15 @@ __device__ __forceinline__ void zm_tile(const Geo32& geo, const typename StepV<P
     }
     if (NS == 3) __syncthreads();
   }
+  return true;
 }
 
-// grid: (ceil(nx / ZM_TX), ceil(ny / TY), ceil(nz / zc)), block ZM_TX x TY with
-// TY = zm_ty(FLAT).
+// grid: (ceil(nx / TX), ceil(ny / TY), ceil(nz / zc)), block TX x TY.
 // tclock (launches replayed from a CUDA graph): the FP16 rounding seed comes
 // from the step count *tclock + tofs in device memory instead of `seed`, the
 // same function of the step count as the host's.
-template <int PREC, int QH, int FLAT, int SOLID = 0>
-__global__ void __launch_bounds__(ZM_TX* zm_ty(FLAT), zm_minb(PREC, ZM_TX* zm_ty(FLAT)))
+template <int PREC, int QH, int FLAT, int SOLID = 0, int TX = ZM_TX, int TY = zm_ty(FLAT)>
+__global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
     k_step_zm(Geo32 geo, typename StepV<PREC>::Par ph, const typename Store<PREC>::S* __restrict__ hA,
               const typename Store<PREC>::S* __restrict__ gA, typename Store<PREC>::S* __restrict__ hB,
               typename Store<PREC>::S* __restrict__ gB, const typename Store<PREC>::PhiT* __restrict__ phi_shift,
@@ -1293,8 +1347,34 @@ __global__ void __launch_bounds__(ZM_TX* zm_ty(FLAT), zm_minb(PREC, ZM_TX* zm_ty
   // global memory only after the previous step has completed
   if (PFL_ZM_PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (PREC == 2 && tclock) seed = step_seed_of(*tclock + (unsigned long long)tofs);
-  zm_tile<PREC, QH, zm_ty(FLAT), FLAT, SOLID>(geo, ph, hA, gA, hB, gB, phi_shift, phi_out, zc, seed, links, pg_in,
-                                              pg_out, blockIdx.x, blockIdx.y, blockIdx.z);
+  zm_tile<PREC, QH, TY, FLAT, SOLID, TX>(geo, ph, hA, gA, hB, gB, phi_shift, phi_out, zc, seed, links, pg_in, pg_out,
+                                         blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+// The same with the populations read by tensor copies (3-D lattices without
+// solid cells whose rows are whole 16-byte units), in tiles of TX x TY.  err: set
+// when a copy did not arrive.
+template <int PREC, int QH, int TX, int TY>
+__global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
+    k_step_tma(const __grid_constant__ StepMaps maps, Geo32 geo, typename StepV<PREC>::Par ph,
+               const typename Store<PREC>::S* __restrict__ hA, const typename Store<PREC>::S* __restrict__ gA,
+               typename Store<PREC>::S* __restrict__ hB, typename Store<PREC>::S* __restrict__ gB,
+               const typename Store<PREC>::PhiT* __restrict__ phi_shift,
+               typename Store<PREC>::PhiT* __restrict__ phi_out, int zc, unsigned seed, const unsigned long long* tclock,
+               int tofs, const __half* __restrict__ pg_in, __half* __restrict__ pg_out, volatile int* err) {
+  __shared__ unsigned long long mbar[2];
+  const unsigned bar = smem_u32(mbar);
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    mbar_init(bar);
+    mbar_init(bar + 8);
+  }
+  __syncthreads();
+  if (PFL_ZM_PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (PREC == 2 && tclock) seed = step_seed_of(*tclock + (unsigned long long)tofs);
+  if (!zm_tile<PREC, QH, TY, 0, 0, TX, 1>(geo, ph, hA, gA, hB, gB, phi_shift, phi_out, zc, seed, nullptr, pg_in, pg_out,
+                                          blockIdx.x, blockIdx.y, blockIdx.z, &maps, bar) &&
+      threadIdx.x == 0 && threadIdx.y == 0)
+    *err = 1;
 }
 
 }  // namespace pfl
