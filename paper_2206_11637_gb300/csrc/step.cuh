@@ -405,9 +405,9 @@ __device__ __forceinline__ Mom<V> moments(const LD& ld) {
 // Moments of an FP16S set: f_i = w_i (s_i / K + shift of its writer), the
 // stored and the shift part summed apart (differences of large shifts cancel
 // exactly) and joined once.
-template <int Q, class V, class LD, class SH>
-__device__ __forceinline__ Mom<V> moments_f16(const LD& ld, const SH& sh, double K) {
-  const Mom<V> a = moments<Q, 1, V>(ld), b = moments<Q, 1, V>(sh);
+template <int Q, class V, class SH>
+__device__ __forceinline__ Mom<V> moments_join(const Mom<V>& a, const SH& sh, double K) {
+  const Mom<V> b = moments<Q, 1, V>(sh);
   const V k = vbc<V>(1.0 / K), n = vbc<V>(1.0 / wsum_of<Q>());
   Mom<V> m;
   m.s = vfma(k, a.s, b.s) * n;
@@ -454,20 +454,27 @@ __device__ __forceinline__ Mom<F1> moments_pairs(const LD& ld) {
 template <int PREC, int QH, class V, class LD, class SH>
 __device__ __forceinline__ Mom<V> h_moments(const LD& ld, const SH& sh) {
   if constexpr (PREC == 2)
-    return moments_f16<QH, V>(ld, sh, KH16);
+    return moments_join<QH, V>(moments<QH, 1, V>(ld), sh, KH16);
   else if constexpr (PREC == 1)
     return moments_pairs<QH>(ld);
   else
     return moments<QH, 0, V>(ld);
 }
-template <int PREC, int QG, class V, class LD, class SH>
-__device__ __forceinline__ Mom<V> g_moments(const LD& ld, const SH& sh) {
-  if constexpr (PREC == 2)
-    return moments_f16<QG, V>(ld, sh, KG16);
-  else if constexpr (PREC == 1)
+// The g moments in two parts: of the stored values, and (FP16S) joined with the
+// p* shifts.
+template <int PREC, int QG, class V, class LD>
+__device__ __forceinline__ Mom<V> g_moments_stored(const LD& ld) {
+  if constexpr (PREC == 1)
     return moments_pairs<QG>(ld);
   else
-    return moments<QG, 0, V>(ld);
+    return moments<QG, PREC == 2, V>(ld);
+}
+template <int PREC, int QG, class V, class SH>
+__device__ __forceinline__ Mom<V> g_moments_shift(const Mom<V>& a, const SH& sh) {
+  if constexpr (PREC == 2)
+    return moments_join<QG, V>(a, sh, KG16);
+  else
+    return a;
 }
 
 // ---------------------------------------------------------------------------
@@ -997,8 +1004,9 @@ __device__ __forceinline__ void step_cell(const Geo32& geo, const typename StepV
   CellOff o;
   cell_off(geo, cell, o);
   auto at = [&](int cx, int cy, int cz) { return (R)__ldg(phi + cell + o.soff(cx, cy, cz)); };
-  const Mom<V> gm = g_moments<PREC, QG, V>(
-      [&](int cx, int cy, int cz) { return V{load_dir<PREC, QG, ODD>(g, geo.N, cell, o, cx, cy, cz)}; },
+  const Mom<V> gm = g_moments_shift<PREC, QG, V>(
+      g_moments_stored<PREC, QG, V>(
+          [&](int cx, int cy, int cz) { return V{load_dir<PREC, QG, ODD>(g, geo.N, cell, o, cx, cy, cz)}; }),
       [&](int cx, int cy, int cz) { return V{(R)__half2float(__ldg(pg_in + writer(cell, o, cx, cy, cz)))}; });
   CellOut<PREC, QH, ODD> out{h, g, geo.N, cell, o, pg_out, Dither{PREC == 2 ? hash32(cell * 0x9E3779B1u + seed) : 0u}};
   auto hm = [&] { return h_moments_cell<PREC, QH, ODD>(geo.N, h, shift, cell, o); };
@@ -1143,6 +1151,12 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
   constexpr bool MARCH = PREC != 1 && !SOLID;
   constexpr int NS = FLAT ? 1 : (MARCH ? 2 : (sizeof(R) == 8 ? 3 : 4));
   constexpr int NSP = FLAT ? 1 : 4;
+  // FP32 gathers the g populations of the plane about to collide before the next
+  // plane's h: both sets of loads are in flight together (bubble 186x378x153, no
+  // copies: 13.9 -> 14.5 GLUPS), and with copies one barrier per plane frees both
+  // buffers.  FP16S (15.6 -> 14.3), single planes (12.5 -> 12.2) and solid cells
+  // (Taylor tube 66x640x66: 9.7 -> 9.6) lose by it.
+  constexpr bool EARLY = PREC == 1 && !FLAT && !SOLID;
   __shared__ PhiT ring[NS][PS];
   __shared__ V hmom[FLAT ? 1 : 2][10 * NT];
   __shared__ float pring[F16 ? NSP : 1][F16 ? PS : 1];  // FP16S: p* shifts of the stored g, ring like phi
@@ -1236,22 +1250,25 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
     return phi_plane<V>([&](int cx, int cy) { return V{(R)ring[slot][i0 + cy * PW + cx]}; });
   };
 
-  // g moments of the own cell of plane z (plane count b)
+  // g moments of the own cell of plane z (plane count b): the stored values,
+  // then the p* shifts
   unsigned cell = 0;
   CellOff o;
-  Mom<V> gm;
-  auto gather_g = [&](int b) {
-    gm = g_moments<PREC, QG, V>(
-        [&](int cx, int cy, int cz) {
-          const unsigned i = (unsigned)lq_index<QG>(cx, cy, cz);
-          if constexpr (TM != 0) return V{raw<PREC>(sG[i * NT + tid])};
-          return V{raw<PREC>(gA[i * N + cell])};
-        },
-        [&](int cx, int cy, int cz) {  // p* of the writer x - c, or of the cell itself after a bounce-back
-          const float* p0 = pring[FLAT ? 0 : b % NSP];
-          const float* pz = FLAT ? p0 : pring[(b - cz) % NSP];
-          return V{o.valid(-cx, -cy, -cz) ? (R)pz[i0 - cy * PW - cx] : (R)p0[i0]};
-        });
+  Mom<V> gm = {};
+  auto gather_g = [&] {
+    gm = g_moments_stored<PREC, QG, V>([&](int cx, int cy, int cz) {
+      const unsigned i = (unsigned)lq_index<QG>(cx, cy, cz);
+      if constexpr (TM != 0) return V{raw<PREC>(sG[i * NT + tid])};
+      return V{raw<PREC>(gA[i * N + cell])};
+    });
+  };
+  auto shift_g = [&](int b) {
+    gm = g_moments_shift<PREC, QG, V>(gm, [&](int cx, int cy, int cz) {
+      // p* of the writer x - c, or of the cell itself after a bounce-back
+      const float* p0 = pring[FLAT ? 0 : b % NSP];
+      const float* pz = FLAT ? p0 : pring[(b - cz) % NSP];
+      return V{o.valid(-cx, -cy, -cz) ? (R)pz[i0 - cy * PW - cx] : (R)p0[i0]};
+    });
   };
 
   // Planes z0 - 1 .. z1 are filled in turn; once plane z + 1 is, plane z
@@ -1262,12 +1279,9 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
   for (int zp = FLAT ? z0 : z0 - 1; zp <= (FLAT ? z0 : z1); ++zp) {
     const int z = FLAT ? zp : zp - 1;
     const int bp = zp - (z0 - 1), b = bp - 1;  // plane counts from z0 - 1
-    // FP32 gathers g before the barrier, so that one barrier frees both copies;
-    // FP16S needs the p* shifts of plane z + 1 first
-    if (TM && !F16 && z >= z0) {
-      ok = mbar_wait(mbar + 8, phase_g++ & 1) && ok;
-      gather_g(b);
-    }
+    cell = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)z);
+    if (TM && z >= z0) ok = mbar_wait(mbar + 8, phase_g++ & 1) && ok;
+    if (EARLY && z >= z0 && (TM || active)) gather_g();
     fill(FLAT ? 0 : zp, FLAT ? 0 : bp % NS, FLAT ? 0 : bp % NSP, FLAT ? 0 : bp & 1);
     if constexpr (TM != 0) {
       if (!__syncthreads_and(ok)) {
@@ -1277,7 +1291,7 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
         return false;
       }
       if (zp < z1) issue_h(zp + 1);
-      if (zp < z1 && (F16 ? zp == z0 : zp >= z0)) issue_g(zp);
+      if (zp < z1 && zp >= z0) issue_g(zp);
     } else {
       __syncthreads();
     }
@@ -1288,21 +1302,15 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
       po = pp;
       continue;
     }
-    cell = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)z);
     const unsigned blk = (SOLID && active) ? __ldg(links + cell) : 0u;
     o = off_xyz(geo, (unsigned)x, (unsigned)y, (unsigned)z, blk);
-    if (TM && F16) {
-      ok = mbar_wait(mbar + 8, phase_g++ & 1) && ok;
-      gather_g(b);
-      __syncthreads();
-      if (z + 1 < z1) issue_g(z + 1);
-    }
     if (SOLID && active && (blk & SOLID_SELF)) {
       phi_out[cell] = (PhiT)0;  // solid cells are not updated; their populations stay zero
     } else if (active) {
       const PhiT* at0 = ring[FLAT ? 0 : b % NS];
       phi_out[cell] = at0[i0];
-      if (!TM) gather_g(b);
+      if (!EARLY) gather_g();
+      shift_g(b);
       CellOut<PREC, QH, 1> out{hB, gB, N, cell, o, pg_out, Dither{F16 ? hash32(cell * 0x9E3779B1u + seed) : 0u}};
       const V* hp = &hmom[FLAT ? 0 : b & 1][tid];
       auto hm = [&] {
