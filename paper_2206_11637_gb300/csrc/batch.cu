@@ -246,11 +246,22 @@ const void* batch_fn(int j) {
   return nullptr;
 }
 
+// (Launched with programmatic stream serialisation, as the single-lattice step:
+// a block waits for the previous grid before its first global access, and that
+// grid had waited for its own predecessor, the class's last step.)
 template <int PREC, int CLS, int J>
 void launch_shape(pfl_batch* b, const ClassPlan& c) {
-  k_batch_zm<PREC, SHAPES[CLS][J][0], SHAPES[CLS][J][1], CLS == 0>
-      <<<c.shape.grid, dim3(SHAPES[CLS][J][0], SHAPES[CLS][J][1]), 0, b->stream>>>(
-          b->d_inst, c.tiles, c.ntiles, b->ab, (unsigned*)(b->ws + b->ctr_off) + 2 * CLS);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3(c.shape.grid);
+  cfg.blockDim = dim3(SHAPES[CLS][J][0], SHAPES[CLS][J][1]);
+  cfg.stream = b->stream;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = PFL_ZM_PDL ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k_batch_zm<PREC, SHAPES[CLS][J][0], SHAPES[CLS][J][1], CLS == 0>, (const BInst*)b->d_inst,
+                     (const BTile*)c.tiles, c.ntiles, b->ab, (unsigned*)(b->ws + b->ctr_off) + 2 * CLS);
 }
 
 template <int PREC, int CLS>
@@ -677,11 +688,7 @@ pfl_status pfl_batch_fields(pfl_batch* b, int i, double* phi, double* rho, doubl
   BTRY(cudaGetLastError());
   double* want[6] = {phi, rho, p, u, u ? u + N : nullptr, u ? u + 2 * N : nullptr};
   double* st = (double*)(b->ws + b->stage_off);
-  for (int k = 0; k < 6; ++k) {
-    if (!want[k]) continue;
-    const bool dev = is_device_ptr(want[k]);
-    double* o[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    o[k] = dev ? want[k] : st;
+  auto launch = [&](double* const o[6]) {
     const unsigned nb = blocks_for(N, 256);
     if (b->prec == PFL_FP64)
       k_fields<0, 15, 0><<<nb, 256, 0, b->stream>>>(geo, I.ph, (const Store<0>::S*)I.g[ab], (const Store<0>::PhiT*)I.phic,
@@ -689,10 +696,27 @@ pfl_status pfl_batch_fields(pfl_batch* b, int i, double* phi, double* rho, doubl
     else
       k_fields<1, 15, 0><<<nb, 256, 0, b->stream>>>(geo, I.ph, (const Store<1>::S*)I.g[ab], (const Store<1>::PhiT*)I.phic,
                                                     o[0], o[1], o[2], o[3], o[4], o[5]);
+  };
+  // device outputs in one pass, host outputs one at a time through the staging area
+  double* dev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  bool any_dev = false;
+  for (int k = 0; k < 6; ++k)
+    if (is_device_ptr(want[k])) {
+      dev[k] = want[k];
+      any_dev = true;
+    }
+  if (any_dev) launch(dev);
+  BTRY(cudaGetLastError());
+  for (int k = 0; k < 6; ++k) {
+    if (!want[k] || dev[k]) continue;
+    double* o[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    o[k] = st;
+    launch(o);
     BTRY(cudaGetLastError());
-    if (!dev) BTRY(cudaMemcpyAsync(want[k], st, N * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+    BTRY(cudaMemcpyAsync(want[k], st, N * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
     BTRY(cudaStreamSynchronize(b->stream));
   }
+  BTRY(cudaStreamSynchronize(b->stream));
   return PFL_OK;
 }
 
