@@ -98,6 +98,11 @@ Layout layout_of(const pfl_params* p) {
 
 }  // namespace
 
+// cuTensorMapEncodeTiled, looked up at run time (the library links no driver stub)
+typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
 struct pfl_ctx {
   pfl_params p;
   Geo geo;
@@ -132,6 +137,7 @@ struct pfl_ctx {
   // kernel reports to when a copy did not arrive
   int tma;
   StepMaps maps[2];
+  EncodeTiled encode;
   int* err;
   bool wide;     // fused step without copies in tiles of WIDE_TX x WIDE_TY
 };
@@ -264,10 +270,6 @@ constexpr int TMA_TILES[NTMA][2] = {{128, 2}, {64, 4}};
 constexpr int TMA_ZC = 12;
 constexpr long long TMA_CELLS = 1 << 19;
 
-typedef CUresult (*EncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 // The kernel of a tile, its dynamic shared memory and, on request, its launch.
 template <int PREC, int QH, int J>
 struct TmaStep {
@@ -321,28 +323,27 @@ int tma_tile(const pfl_params* p) {
   return best;
 }
 
-// Tensor maps of the two array pairs, launch attributes, the error word and the
-// z chunk of a context that takes tile shape c->tma.
+// Tensor maps of the pair (h, g) for the context's tile.
+bool make_maps(const pfl_ctx* c, StepMaps* m, void* h, void* g) {
+  const cuuint64_t S = pop_bytes(c->p.precision), nx = c->p.nx, ny = c->p.ny, nz = c->p.nz, N = nx * ny * nz;
+  auto make = [&](CUtensorMap* map, void* base, cuuint32_t q) {
+    const cuuint64_t dims[4] = {nx, ny, nz, q}, strides[3] = {nx * S, nx * ny * S, N * S};
+    const cuuint32_t box[4] = {(cuuint32_t)TMA_TILES[c->tma][0], (cuuint32_t)TMA_TILES[c->tma][1], 1, q}, es[4] = {1, 1, 1, 1};
+    return c->encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+           CUDA_SUCCESS;
+  };
+  return make(&m->h, h, (cuuint32_t)c->qh) && make(&m->g, g, (cuuint32_t)c->qg);
+}
+
+// Launch attributes and the z chunk of a context that takes tile shape c->tma.
 template <int PREC, int QH>
-void setup_tma_t(pfl_ctx* c, EncodeTiled enc, int sms, bool* ok) {
+void setup_tma_t(pfl_ctx* c, int sms, bool* ok) {
   if constexpr (has_tma<PREC, QH>()) {
     const int tx = TMA_TILES[c->tma][0], ty = TMA_TILES[c->tma][1];
-    const cuuint64_t S = sizeof(typename Store<PREC>::S), nx = c->p.nx, ny = c->p.ny, nz = c->p.nz, N = nx * ny * nz;
-    auto make = [&](CUtensorMap* m, size_t off, cuuint32_t q) {
-      const cuuint64_t dims[4] = {nx, ny, nz, q}, strides[3] = {nx * S, nx * ny * S, N * S};
-      const cuuint32_t box[4] = {(cuuint32_t)tx, (cuuint32_t)ty, 1, q}, es[4] = {1, 1, 1, 1};
-      return enc(m, PREC == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, c->ws + off, dims, strides,
-                 box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    };
-    *ok = make(&c->maps[0].h, c->L.h, QH) && make(&c->maps[0].g, c->L.g, 27) && make(&c->maps[1].h, c->L.h2, QH) &&
-          make(&c->maps[1].g, c->L.g2, 27);
     int per_sm = 1;
     tma_shape<PREC, QH>(c->tma, [&](auto k) { *ok = *ok && k.prepare(&per_sm); });
-    *ok = *ok && per_sm > 0 && cudaHostAlloc((void**)&c->err, 64, cudaHostAllocPortable) == cudaSuccess;
-    if (!*ok) return;
-    *c->err = 0;
-    const long long slots = (long long)sms * per_sm;
+    const long long slots = (long long)sms * (per_sm < 1 ? 1 : per_sm);
     const long long blocks = (long long)((c->p.nx + tx - 1) / tx) * ((c->p.ny + ty - 1) / ty) * ((c->p.nz + TMA_ZC - 1) / TMA_ZC);
     // from two waves on the last one's share is small and the march's length counts
     c->zc = blocks >= 2 * slots ? TMA_ZC : z_chunk(&c->p, tx, ty, slots, TMA_ZC);
@@ -597,9 +598,12 @@ bool setup_tma(pfl_ctx* c, int sms) {
   if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
       q != cudaDriverEntryPointSuccess)
     return false;
-  bool ok = true;
-  DISPATCH(c, setup_tma_t, c, (EncodeTiled)fn, sms, &ok);
-  return ok;
+  c->encode = (EncodeTiled)fn;
+  bool ok = make_maps(c, &c->maps[0], c->ws + c->L.h, c->ws + c->L.g) && make_maps(c, &c->maps[1], c->ws + c->L.h2, c->ws + c->L.g2);
+  DISPATCH(c, setup_tma_t, c, sms, &ok);
+  if (!ok || cudaHostAlloc((void**)&c->err, 64, cudaHostAllocPortable) != cudaSuccess) return false;
+  *c->err = 0;
+  return true;
 }
 
 // Releases what the context holds on the host.
@@ -1350,8 +1354,8 @@ pfl_status copy_state(pfl_ctx* c, char* slot, bool save) {
 }
 
 template <int PREC>
-void launch_dot(pfl_ctx* c, const double* W, double* part, double* out) {
-  k_dot<typename Store<PREC>::PhiT><<<DOT_BLOCKS, 256, 0, c->stream>>>((unsigned)c->geo.N, W, phicur<PREC>(c), part);
+void launch_dot(pfl_ctx* c, const double* W, const typename Store<PREC>::PhiT* phi, double* part, double* out) {
+  k_dot<typename Store<PREC>::PhiT><<<DOT_BLOCKS, 256, 0, c->stream>>>((unsigned)c->geo.N, W, phi, part);
   k_sum_parts<<<1, 32, 0, c->stream>>>(part, DOT_BLOCKS, 1, out);
 }
 
@@ -1404,27 +1408,47 @@ struct SlotPtr {
     g = (typename Store<PREC>::S*)(slot + align256(hb));
     phi = (typename Store<PREC>::PhiT*)(slot + align256(hb) + align256((size_t)c->qg * N * S));
   }
+  SlotPtr(typename Store<PREC>::S* h_, typename Store<PREC>::S* g_, typename Store<PREC>::PhiT* phi_) : h(h_), g(g_), phi(phi_) {}
 };
 
-// One fused step from slot a into slot b; phi of a (the sum the kernel forms
-// in shared memory) goes to a's phi.  FP64 / FP32 only: no shifts.
+// One fused step from the state a into the state b; phi of a (the sum the kernel
+// forms in shared memory) goes to a's phi.  FP64 / FP32 only: no shifts.  The
+// tensor maps of a are made for the launch.
 template <int PREC, int QH>
-void zm_step_slots(pfl_ctx* c, const SlotPtr<PREC>& a, const SlotPtr<PREC>& b) {
+pfl_status zm_step_slots(pfl_ctx* c, const SlotPtr<PREC>& a, const SlotPtr<PREC>& b) {
+  const typename StepV<PREC>::Par ph = step_par<PREC>(c->ph);
+  if (c->tma >= 0) {
+    if constexpr (has_tma<PREC, QH>()) {
+      StepMaps m;
+      if (!make_maps(c, &m, a.h, a.g)) return fail(PFL_ERR_CUDA, "encoding the tensor maps of a saved state");
+      cudaLaunchConfig_t cfg = {};
+      cfg.stream = c->stream;
+      tma_shape<PREC, QH>(c->tma, [&](auto k) {
+        k.launch(c, cfg, m, c->g32, ph, (const typename Store<PREC>::S*)a.h, (const typename Store<PREC>::S*)a.g, b.h, b.g,
+                 (const typename Store<PREC>::PhiT*)nullptr, a.phi, c->zc, 0u, (const unsigned long long*)nullptr, 0,
+                 (const __half*)nullptr, (__half*)nullptr, (volatile int*)c->err);
+      });
+    }
+    return PFL_OK;
+  }
   const int ty = zm_ty(c->p.nz == 1);
   const dim3 grid((c->p.nx + ZM_TX - 1) / ZM_TX, (c->p.ny + ty - 1) / ty, (c->p.nz + c->zc_push - 1) / c->zc_push);
   const dim3 block(ZM_TX, ty);
-  const typename StepV<PREC>::Par ph = step_par<PREC>(c->ph);
   if (c->p.nz == 1)
     k_step_zm<PREC, QH, 1><<<grid, block, 0, c->stream>>>(c->g32, ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc_push, 0u);
   else
     k_step_zm<PREC, QH, 0><<<grid, block, 0, c->stream>>>(c->g32, ph, a.h, a.g, b.h, b.g, nullptr, a.phi, c->zc_push, 0u);
+  return PFL_OK;
 }
 
 // Adjoint with the fused two-array engine.  Forward sweep: checkpoints every K
-// steps, phi formed only where a checkpoint or an observation needs it.
-// Reverse sweep, per segment: the checkpoint is copied into slot 0 and each
-// recomputed step writes the next slot directly, so the live state (t_end) is
-// never touched and no per-step copy is made.
+// steps, phi formed only where a checkpoint or an observation needs it.  A state
+// that is a checkpoint is written by its step into the checkpoint's slot and
+// stepped on from there, and the reverse sweep's segments start in that slot:
+// only the first state is ever copied (25 steps of a 128x384x128 FP32 bubble
+// copied ten states of 1.1 GB, 3.3 of 40.4 ms).
+// Reverse sweep, per segment: each recomputed step writes the next slot, so
+// the live state (t_end) is never touched.
 template <int PREC, int QH, class ObsAt>
 pfl_status run_adjoint_zm(pfl_ctx* c, int n, const ObsAt& obs_at, char* aws, const AdjLayout& A, double* J,
                           double grad[3]) {
@@ -1432,18 +1456,43 @@ pfl_status run_adjoint_zm(pfl_ctx* c, int n, const ObsAt& obs_at, char* aws, con
   double* res = (double*)(aws + A.res);
   double* part = (double*)(aws + A.part);
   double* dot_part = part + 3 * ((c->geo.N + ADJ_THREADS - 1) / ADJ_THREADS);
+  const unsigned nbp = blocks_for(c->geo.N, 256);
+  auto ck = [&](int k) { return SlotPtr<PREC>(c, aws + A.ck + (size_t)(k / A.K) * A.state); };
+  auto live = [&](int ab) {
+    return SlotPtr<PREC>((typename Store<PREC>::S*)(c->ws + (ab ? c->L.h2 : c->L.h)),
+                         (typename Store<PREC>::S*)(c->ws + (ab ? c->L.g2 : c->L.g)), phicur<PREC>(c));
+  };
   for (int k = 0; k < n; ++k) {
     const double* W = obs_at(k);
-    if (k % A.K == 0 || W) ensure_phi<PREC, QH>(c);
-    if (k % A.K == 0) {
-      pfl_status s = copy_state(c, aws + A.ck + (size_t)(k / A.K) * A.state, true);
+    const bool in_ck = k > 0 && k % A.K == 0;  // state k sits in its checkpoint
+    if (k == 0) {
+      ensure_phi<PREC, QH>(c);
+      pfl_status s = copy_state(c, aws + A.ck, true);
       if (s != PFL_OK) return s;
     }
-    if (W) launch_dot<PREC>(c, W, dot_part, res);
-    step_only<PREC, QH, 0>(c);
+    if (W) {
+      if (in_ck) {
+        k_phi32<PREC, QH, 0><<<nbp, 256, 0, c->stream>>>(c->g32, ck(k).h, nullptr, ck(k).phi);
+        launch_dot<PREC>(c, W, ck(k).phi, dot_part, res);
+      } else {
+        ensure_phi<PREC, QH>(c);
+        launch_dot<PREC>(c, W, phicur<PREC>(c), dot_part, res);
+      }
+    }
+    const bool to_ck = k + 1 < n && (k + 1) % A.K == 0;
+    if (in_ck || to_ck) {
+      const pfl_status s = zm_step_slots<PREC, QH>(c, in_ck ? ck(k) : live(c->ab), to_ck ? ck(k + 1) : live(c->ab ^ 1));
+      if (s != PFL_OK) return s;
+      c->ab ^= 1;
+      c->cur = 1 - c->cur;
+      c->stale = true;
+      c->t += 1;
+    } else {
+      step_only<PREC, QH, 0>(c);
+    }
   }
   ensure_phi<PREC, QH>(c);
-  if (const double* W = obs_at(n)) launch_dot<PREC>(c, W, dot_part, res);
+  if (const double* W = obs_at(n)) launch_dot<PREC>(c, W, phicur<PREC>(c), dot_part, res);
   CUDA_TRY(cudaGetLastError());
 
   void* lam = aws + A.lam0;
@@ -1454,17 +1503,19 @@ pfl_status run_adjoint_zm(pfl_ctx* c, int n, const ObsAt& obs_at, char* aws, con
                                                                    (R*)(aws + A.acc), obs_at(n));
   for (int sgm = A.nck - 1; sgm >= 0; --sgm) {
     const int k0 = sgm * A.K, k1 = (k0 + A.K < n) ? k0 + A.K : n;
-    char* seg = aws + A.seg;
-    CUDA_TRY(cudaMemcpyAsync(seg, aws + A.ck + (size_t)sgm * A.state, A.state, cudaMemcpyDeviceToDevice, c->stream));
-    for (int k = k0; k + 1 < k1; ++k)
-      zm_step_slots<PREC, QH>(c, SlotPtr<PREC>(c, seg + (size_t)(k - k0) * A.state),
-                          SlotPtr<PREC>(c, seg + (size_t)(k + 1 - k0) * A.state));
-    if (k1 - 1 > k0) {  // phi of the last slot (the others were formed by the steps out of them)
-      const SlotPtr<PREC> last(c, seg + (size_t)(k1 - 1 - k0) * A.state);
-      k_phi32<PREC, QH, 0><<<blocks_for(c->geo.N, 256), 256, 0, c->stream>>>(c->g32, last.h, nullptr, last.phi);
+    // state k of the segment: its first in the checkpoint, the others in their slots
+    auto slot = [&](int k) {
+      return aws + (k == k0 ? A.ck + (size_t)sgm * A.state : A.seg + (size_t)(k - k0) * A.state);
+    };
+    for (int k = k0; k + 1 < k1; ++k) {
+      const pfl_status s = zm_step_slots<PREC, QH>(c, SlotPtr<PREC>(c, slot(k)), SlotPtr<PREC>(c, slot(k + 1)));
+      if (s != PFL_OK) return s;
     }
+    // phi of the last slot (the others were formed by the steps out of them)
+    const SlotPtr<PREC> last(c, slot(k1 - 1));
+    k_phi32<PREC, QH, 0><<<nbp, 256, 0, c->stream>>>(c->g32, last.h, nullptr, last.phi);
     for (int k = k1 - 1; k >= k0; --k) {
-      launch_adj_step<PREC, QH>(c, A, aws, seg + (size_t)(k - k0) * A.state, 0, lam, lam2, obs_at(k));
+      launch_adj_step<PREC, QH>(c, A, aws, slot(k), 0, lam, lam2, obs_at(k));
       std::swap(lam, lam2);
     }
     CUDA_TRY(cudaGetLastError());
@@ -1476,7 +1527,7 @@ pfl_status run_adjoint_zm(pfl_ctx* c, int n, const ObsAt& obs_at, char* aws, con
   if (J) *J = hres[0];
   if (grad)
     for (int k = 0; k < 3; ++k) grad[k] = hres[1 + k];
-  return PFL_OK;
+  return check_err(c);
 }
 
 // The weight field of the observation at step k (relative to the adjoint's
@@ -1523,14 +1574,14 @@ pfl_status run_adjoint(pfl_ctx* c, int n, const ObsTable& obs_at, char* aws, con
       pfl_status s = copy_state(c, aws + A.ck + (size_t)(k / A.K) * A.state, true);
       if (s != PFL_OK) return s;
     }
-    if (const double* W = obs_at(k)) launch_dot<PREC>(c, W, part + 3 * ((c->geo.N + ADJ_THREADS - 1) / ADJ_THREADS), res);
+    if (const double* W = obs_at(k)) launch_dot<PREC>(c, W, phicur<PREC>(c), part + 3 * ((c->geo.N + ADJ_THREADS - 1) / ADJ_THREADS), res);
     const bool bgk = false;
     (void)bgk;
     step_only<PREC, QH, 0>(c);
     after_step<PREC, QH>(c);
     ensure_phi<PREC, QH>(c);
   }
-  if (const double* W = obs_at(n)) launch_dot<PREC>(c, W, part + 3 * ((c->geo.N + ADJ_THREADS - 1) / ADJ_THREADS), res);
+  if (const double* W = obs_at(n)) launch_dot<PREC>(c, W, phicur<PREC>(c), part + 3 * ((c->geo.N + ADJ_THREADS - 1) / ADJ_THREADS), res);
   const int fin_swapped = c->swapped;
   const long long t_end = c->t;
   pfl_status st = copy_state(c, aws + A.fin, true);
