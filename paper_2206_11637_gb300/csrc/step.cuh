@@ -1232,27 +1232,36 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
     float rp = 0;
     if constexpr (RING1ST) ring_cell(NRING < NT ? min(tid, NRING - 1) : tid, rat, rv, rp);
     if constexpr (TM != 0) ok = mbar_wait(mbar, phase_h++ & 1) && ok;
-    const Mom<V> m = h_moments<PREC, QH, V>(
-        [&](int cx, int cy, int cz) {
-          const unsigned i = (unsigned)lq_index<QH>(cx, cy, cz);
-          if constexpr (TM != 0) return V{raw<PREC>(sH[i * NT + tid])};
-          return V{raw<PREC>(hA[i * N + c])};
-        },
-        [&](int cx, int cy, int cz) { return V{(R)__ldg(phi_shift + writer(c, o, cx, cy, cz))}; });
-    // (tile positions outside the lattice serve as ring cells; the copy does not hold them)
-    ring[slot][i0] = TM && !active ? phi_at(xq, yq, zq) : (PhiT)m.s.v;
+    if (PREC == 0 && !FLAT && (zp < z0 || zp >= z1)) {
+      // FP64, the planes beside the chunk: their cells collide in other blocks, so
+      // phi alone (14 additions instead of 39): drop 32^3, one plane per chunk,
+      // 47.7 -> 43.9 us per step, 64^3 295 -> 288, bubble 61x183x61 742 -> 728, D3Q27
+      // drop 48^3 190 -> 178.  FP32 and FP16S do not wait for the additions and
+      // lose 3 % by the second code site.
+      ring[slot][i0] = phi_at(xq, yq, zq);
+    } else {
+      const Mom<V> m = h_moments<PREC, QH, V>(
+          [&](int cx, int cy, int cz) {
+            const unsigned i = (unsigned)lq_index<QH>(cx, cy, cz);
+            if constexpr (TM != 0) return V{raw<PREC>(sH[i * NT + tid])};
+            return V{raw<PREC>(hA[i * N + c])};
+          },
+          [&](int cx, int cy, int cz) { return V{(R)__ldg(phi_shift + writer(c, o, cx, cy, cz))}; });
+      // (tile positions outside the lattice serve as ring cells; the copy does not hold them)
+      ring[slot][i0] = TM && !active ? phi_at(xq, yq, zq) : (PhiT)m.s.v;
+      V* hm = &hmom[mslot][tid];
+      hm[0] = m.s;
+      hm[NT] = m.x;
+      hm[2 * NT] = m.y;
+      hm[3 * NT] = m.z;
+      hm[4 * NT] = m.xx;
+      hm[5 * NT] = m.yy;
+      hm[6 * NT] = m.zz;
+      hm[7 * NT] = m.xy;
+      hm[8 * NT] = m.yz;
+      hm[9 * NT] = m.xz;
+    }
     if constexpr (F16) pring[pslot][i0] = ld_pshift(pg_in, c);
-    V* hm = &hmom[mslot][tid];
-    hm[0] = m.s;
-    hm[NT] = m.x;
-    hm[2 * NT] = m.y;
-    hm[3 * NT] = m.z;
-    hm[4 * NT] = m.xx;
-    hm[5 * NT] = m.yy;
-    hm[6 * NT] = m.zz;
-    hm[7 * NT] = m.xy;
-    hm[8 * NT] = m.yz;
-    hm[9 * NT] = m.xz;
     if (RING1ST && tid < NRING) ring[slot][rat] = rv;
 #pragma unroll
     for (int r0 = RING1ST ? NT : 0; r0 < NRING; r0 += NT) {
