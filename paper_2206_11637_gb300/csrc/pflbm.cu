@@ -238,6 +238,33 @@ int z_chunk(const pfl_params* p, int tx, int ty, long long slots, int most) {
   return best;
 }
 
+// The same for FP16S on small lattices, whose few blocks leave the SMs unevenly
+// loaded.  The step is bound by what an SM issues, so what counts is the most
+// planes any one SM gets: ceil(blocks / SMs) blocks of zc planes and 0.4 for the
+// two beside them; where fewer than all resident blocks are left, less latency is
+// hidden (one block 1.4, two of three 2.2: 96^3 takes 66 us in 8 planes, three
+// blocks per SM, and 72 us in 12, two).  Against waves of all slots, us per step:
+// drop 64^3 27.8 (3 planes) -> 25.3 (4), 80^3 49.9 (6) -> 46.5 (8); 29^3, 41^3, 50^3,
+// 88^3 and 96^3 keep their planes.
+// Lattices of many rounds keep the waves: a 6.3 M-cell bubble 15.6 GLUPS at
+// their 19 planes, 15.3 at the 12 this count gives.
+constexpr long long SMALL_CELLS = 1 << 20;
+int z_chunk_small(const pfl_params* p, int tx, int ty, long long sms, int resident) {
+  const long long bxy = (long long)((p->nx + tx - 1) / tx) * ((p->ny + ty - 1) / ty);
+  int best = p->nz;
+  double best_cost = 1e300;
+  for (int zc = best; zc >= 1; --zc) {
+    const long long per_sm = (bxy * ((p->nz + zc - 1) / zc) + sms - 1) / sms;
+    const long long rest = per_sm % resident;
+    const double cost = (per_sm + (rest == 0 ? 0.0 : rest == 1 ? 0.4 : 0.2)) * (zc + 0.4);
+    if (cost < best_cost * (1 - 1e-9)) {
+      best_cost = cost;
+      best = zc;
+    }
+  }
+  return best;
+}
+
 // share of the threads of tx x ty tiles that hold a cell
 double tile_use(const pfl_params* p, int tx, int ty) {
   auto part = [](int n, int t) { return (double)n / ((n + t - 1) / t * t); };
@@ -801,6 +828,8 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
     else
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_zm<2, 15, 0>, ZM_TX * ZM_TY, 0);
     c->zc_push = c->zc = z_chunk(p, ZM_TX, ZM_TY, (long long)sms * (per_sm < 1 ? 1 : per_sm), p->nz);
+    if (p->precision == PFL_FP16S && p->nz > 1 && (long long)p->nx * p->ny * p->nz <= SMALL_CELLS)
+      c->zc = z_chunk_small(p, ZM_TX, ZM_TY, sms, per_sm < 1 ? 1 : per_sm);
     c->tma = tma_tile(p);
     c->wide = c->tma < 0 && wide_tile(p);
     if (c->wide) c->zc = z_chunk(p, WIDE_TX, WIDE_TY, (long long)sms * PFL_ZM_MINB, p->nz);
