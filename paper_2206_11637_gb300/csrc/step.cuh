@@ -1337,6 +1337,21 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
     } else if (active) {
       const PhiT* at0 = ring[FLAT ? 0 : b % NS];
       phi_out[cell] = at0[i0];
+      // phi around the cell; a solid neighbour reads as the cell itself (neutral wetting)
+      auto at = [&](int cx, int cy, int cz) {
+        if (blk & link_bit(cx, cy, cz)) return (R)at0[i0];
+        return (R)(FLAT ? at0 : ring[(b + cz) % NS])[i0 + cy * PW + cx];
+      };
+      // solid cells: the stencil before g, whose moments then hold no registers
+      // meanwhile (FP16S Taylor tube 62x600x62: 217 -> 206 us per step)
+      V sc = {};
+      Grad<V> sgr = {};
+      if constexpr (PREC != 1 && !MARCH) {
+        auto splane = [&](int cz) { return phi_plane<V>([&](int cx, int cy) { return V{at(cx, cy, cz)}; }); };
+        const PhiPlane<V> p0 = splane(0);
+        sc = p0.c;
+        sgr = QG == 9 ? phi_grad_flat(p0) : phi_grad(splane(-1), p0, splane(1));
+      }
       if (!EARLY) gather_g();
       shift_g(b);
       CellOut<PREC, QH, 1> out{hB, gB, N, cell, o, pg_out, Dither{F16 ? hash32(cell * 0x9E3779B1u + seed) : 0u}};
@@ -1344,19 +1359,12 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
       auto hm = [&] {
         return Mom<V>{hp[0], hp[NT], hp[2 * NT], hp[3 * NT], hp[4 * NT], hp[5 * NT], hp[6 * NT], hp[7 * NT], hp[8 * NT], hp[9 * NT]};
       };
-      // phi around the cell; a solid neighbour reads as the cell itself (neutral wetting)
-      auto at = [&](int cx, int cy, int cz) {
-        if (blk & link_bit(cx, cy, cz)) return (R)at0[i0];
-        return (R)(FLAT ? at0 : ring[(b + cz) % NS])[i0 + cy * PW + cx];
-      };
       if constexpr (PREC == 1) {
         collide_pairs<QH>(ph, at, gm, hm, out);
       } else if constexpr (MARCH) {
         collide<PREC, QH, V>(ph, po.c, FLAT ? phi_grad_flat(po) : phi_grad(pm, po, pp), gm, hm, out);
       } else {
-        auto splane = [&](int cz) { return phi_plane<V>([&](int cx, int cy) { return V{at(cx, cy, cz)}; }); };
-        const PhiPlane<V> p0 = splane(0);
-        collide<PREC, QH, V>(ph, p0.c, QG == 9 ? phi_grad_flat(p0) : phi_grad(splane(-1), p0, splane(1)), gm, hm, out);
+        collide<PREC, QH, V>(ph, sc, sgr, gm, hm, out);
       }
     }
     if (!FLAT) {
