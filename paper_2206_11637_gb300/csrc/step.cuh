@@ -286,18 +286,11 @@ __device__ __forceinline__ void load_pair(const typename Store<PREC>::S* __restr
 // corner part (D3Q15), so the moments up to second order fall out of sums and
 // differences along x, then y, then z: 66 operations for the ten moments of
 // D3Q27 against 111 by opposite pairs, 39 against 63 for D3Q15.
-// ld(cx, cy, cz) gives the population of direction c.  W = 0: populations as
-// they are; W = 1: values divided by their lattice weight, summed with the
-// weights times 216 (D3Q27: (1, 4, 1) per axis), 36 (D2Q9) or 72 (D3Q15: corners
-// 1, axes 8, rest 16), exact multiples.
+// ld(cx, cy, cz) gives the population of direction c.
 template <class V>
 struct Mom {
   V s, x, y, z, xx, yy, zz, xy, yz, xz;  // sum f, sum c f, sum c c f
 };
-template <int Q>
-__host__ __device__ constexpr double wsum_of() {
-  return Q == 27 ? 216.0 : (Q == 9 ? 36.0 : 72.0);
-}
 // index of direction c in the lattice's order
 template <int Q>
 __host__ __device__ constexpr int lq_index(int cx, int cy, int cz) {
@@ -305,55 +298,52 @@ __host__ __device__ constexpr int lq_index(int cx, int cy, int cz) {
   return Q == 27 ? i : (Q == 9 ? i - 9 : (i < 13 ? i / 2 : (i == 13 ? 7 : i / 2 + 1)));
 }
 
-template <int W, class V>
-__device__ __forceinline__ V sum3(V a, V b, V c) {  // a + b + c, or a + 4 b + c
-  if constexpr (W)
-    return vfma(vbc<V>(4.0), b, a + c);
-  else
-    return (a + c) + b;
+template <class V>
+__device__ __forceinline__ V sum3(V a, V b, V c) {
+  return (a + c) + b;
 }
 
 template <class V>
 struct PlaneMom {
   V m00, m10, m20, m01, m11, m02;  // x-order, y-order within one z plane
 };
-template <int W, class V, class LD>
+template <class V, class LD>
 __device__ __forceinline__ PlaneMom<V> plane_mom(const LD& ld, int cz) {
   V a0[3], a1[3], a2[3];
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     const V l = ld(-1, j - 1, cz), c = ld(0, j - 1, cz), r = ld(1, j - 1, cz);
-    a0[j] = sum3<W>(l, c, r);
+    a0[j] = sum3(l, c, r);
     a1[j] = r - l;
     a2[j] = l + r;
   }
   PlaneMom<V> p;
-  p.m00 = sum3<W>(a0[0], a0[1], a0[2]);
+  p.m00 = sum3(a0[0], a0[1], a0[2]);
   p.m01 = a0[2] - a0[0];
   p.m02 = a0[0] + a0[2];
-  p.m10 = sum3<W>(a1[0], a1[1], a1[2]);
+  p.m10 = sum3(a1[0], a1[1], a1[2]);
   p.m11 = a1[2] - a1[0];
-  p.m20 = sum3<W>(a2[0], a2[1], a2[2]);
+  p.m20 = sum3(a2[0], a2[1], a2[2]);
   return p;
 }
 
-template <int Q, int W, class V, class LD>
+template <int Q, class V, class LD>
 __device__ __forceinline__ Mom<V> moments(const LD& ld) {
   Mom<V> m;
   if constexpr (Q == 27) {
-    const PlaneMom<V> a = plane_mom<W, V>(ld, -1), b = plane_mom<W, V>(ld, 0), c = plane_mom<W, V>(ld, 1);
-    m.s = sum3<W>(a.m00, b.m00, c.m00);
+    const PlaneMom<V> a = plane_mom<V>(ld, -1), b = plane_mom<V>(ld, 0), c = plane_mom<V>(ld, 1);
+    m.s = sum3(a.m00, b.m00, c.m00);
     m.z = c.m00 - a.m00;
     m.zz = a.m00 + c.m00;
-    m.x = sum3<W>(a.m10, b.m10, c.m10);
+    m.x = sum3(a.m10, b.m10, c.m10);
     m.xz = c.m10 - a.m10;
-    m.y = sum3<W>(a.m01, b.m01, c.m01);
+    m.y = sum3(a.m01, b.m01, c.m01);
     m.yz = c.m01 - a.m01;
-    m.xx = sum3<W>(a.m20, b.m20, c.m20);
-    m.yy = sum3<W>(a.m02, b.m02, c.m02);
-    m.xy = sum3<W>(a.m11, b.m11, c.m11);
+    m.xx = sum3(a.m20, b.m20, c.m20);
+    m.yy = sum3(a.m02, b.m02, c.m02);
+    m.xy = sum3(a.m11, b.m11, c.m11);
   } else if constexpr (Q == 9) {
-    const PlaneMom<V> b = plane_mom<W, V>(ld, 0);
+    const PlaneMom<V> b = plane_mom<V>(ld, 0);
     m.s = b.m00;
     m.x = b.m10;
     m.y = b.m01;
@@ -377,49 +367,17 @@ __device__ __forceinline__ Mom<V> moments(const LD& ld) {
             zp = ld(0, 0, 1), r = ld(0, 0, 0);
     const V sx = xm + xp, sy = ym + yp, sz = zm + zp, dx = xp - xm, dy = yp - ym, dz = zp - zm;
     const V cx = p[0].m10 + p[1].m10, cy = p[0].m01 + p[1].m01, cz = p[1].m00 - p[0].m00;
-    if constexpr (W) {
-      const V w8 = vbc<V>(8.0);
-      m.s = vfma(vbc<V>(16.0), r, vfma(w8, (sx + sy) + sz, c0));
-      m.x = vfma(w8, dx, cx);
-      m.y = vfma(w8, dy, cy);
-      m.z = vfma(w8, dz, cz);
-      m.xx = vfma(w8, sx, c0);
-      m.yy = vfma(w8, sy, c0);
-      m.zz = vfma(w8, sz, c0);
-    } else {
-      m.s = (c0 + ((sx + sy) + sz)) + r;
-      m.x = cx + dx;
-      m.y = cy + dy;
-      m.z = cz + dz;
-      m.xx = c0 + sx;
-      m.yy = c0 + sy;
-      m.zz = c0 + sz;
-    }
+    m.s = (c0 + ((sx + sy) + sz)) + r;
+    m.x = cx + dx;
+    m.y = cy + dy;
+    m.z = cz + dz;
+    m.xx = c0 + sx;
+    m.yy = c0 + sy;
+    m.zz = c0 + sz;
     m.xy = p[0].m11 + p[1].m11;
     m.xz = p[1].m10 - p[0].m10;
     m.yz = p[1].m01 - p[0].m01;
   }
-  return m;
-}
-
-// Moments of an FP16S set: f_i = w_i (s_i / K + shift of its writer), the
-// stored and the shift part summed apart (differences of large shifts cancel
-// exactly) and joined once.
-template <int Q, class V, class SH>
-__device__ __forceinline__ Mom<V> moments_join(const Mom<V>& a, const SH& sh, double K) {
-  const Mom<V> b = moments<Q, 1, V>(sh);
-  const V k = vbc<V>(1.0 / K), n = vbc<V>(1.0 / wsum_of<Q>());
-  Mom<V> m;
-  m.s = vfma(k, a.s, b.s) * n;
-  m.x = vfma(k, a.x, b.x) * n;
-  m.y = vfma(k, a.y, b.y) * n;
-  m.z = vfma(k, a.z, b.z) * n;
-  m.xx = vfma(k, a.xx, b.xx) * n;
-  m.yy = vfma(k, a.yy, b.yy) * n;
-  m.zz = vfma(k, a.zz, b.zz) * n;
-  m.xy = vfma(k, a.xy, b.xy) * n;
-  m.yz = vfma(k, a.yz, b.yz) * n;
-  m.xz = vfma(k, a.xz, b.xz) * n;
   return m;
 }
 
@@ -447,34 +405,52 @@ __device__ __forceinline__ Mom<F1> moments_pairs(const LD& ld) {
   return Mom<F1>{F1{s}, F1{x}, F1{y}, F1{z}, F1{xx}, F1{yy}, F1{zz}, F1{xy}, F1{yz}, F1{xz}};
 }
 
-// The h moments of a cell (ld: raw stored values, sh: the phi shift of each
-// population's writer, read for FP16S only); m.s is phi.  Everything that
-// forms phi goes through here (a caller that uses m.s alone leaves the rest to
-// dead-code elimination), so all phi of a state agree bitwise.
-template <int PREC, int QH, class V, class LD, class SH>
-__device__ __forceinline__ Mom<V> h_moments(const LD& ld, const SH& sh) {
+// FP16S moments, f_i = w_i (s_i / K + shift of its writer), by opposite pairs in
+// the same order: the stored and the shift part of a pair's sum and difference
+// are formed apart (the difference of two near shifts is exact), joined once, and
+// weighted by the fused multiply-add of each moment.
+template <int Q, class LD, class SH>
+__device__ __forceinline__ Mom<F1> moments_shifted(const LD& ld, const SH& sh, double K) {
+  const F1 k = vbc<F1>(1.0 / K);
+  Mom<F1> m = {};
+  const F1 rest = vfma(ld(0, 0, 0), k, sh(0, 0, 0));
+  bool fx = true, fy = true, fz = true, fxy = true, fyz = true, fxz = true;  // first term of a moment
+  auto add = [](bool& first, F1& acc, F1 w, F1 t) {
+    acc = first ? w * t : vfma(w, t, acc);
+    first = false;
+  };
+#pragma unroll
+  for (int i = 0; i < (Q - 1) / 2; ++i) {
+    const int cx = q27_cx(lq_to27<Q>(i)), cy = q27_cy(lq_to27<Q>(i)), cz = q27_cz(lq_to27<Q>(i));
+    const F1 a = ld(cx, cy, cz), b = ld(-cx, -cy, -cz), pa = sh(cx, cy, cz), pb = sh(-cx, -cy, -cz);
+    const F1 w = vbc<F1>(lq_w<Q>(i)), S = vfma(a + b, k, pa + pb), D = vfma(a - b, k, pa - pb);
+    m.s = i ? vfma(w, S, m.s) : vfma(vbc<F1>(lq_w<Q>((Q - 1) / 2)), rest, w * S);
+    if (cx) m.xx = fx ? w * S : vfma(w, S, m.xx);
+    if (cy) m.yy = fy ? w * S : vfma(w, S, m.yy);
+    if (cz) m.zz = fz ? w * S : vfma(w, S, m.zz);
+    if (cx) add(fx, m.x, cx > 0 ? w : -w, D);
+    if (cy) add(fy, m.y, cy > 0 ? w : -w, D);
+    if (cz) add(fz, m.z, cz > 0 ? w : -w, D);
+    if (cx && cy) add(fxy, m.xy, cx * cy > 0 ? w : -w, S);
+    if (cy && cz) add(fyz, m.yz, cy * cz > 0 ? w : -w, S);
+    if (cx && cz) add(fxz, m.xz, cx * cz > 0 ? w : -w, S);
+  }
+  return m;
+}
+
+// The moments of a set of a cell: ld gives the raw stored value arriving by
+// direction c, sh (FP16S; K the format's factor) the shift of its writer.  m.s is
+// phi (h) or p* (g).  Everything that forms phi goes through here (a caller that
+// uses m.s alone leaves the rest to dead-code elimination), so all phi of a
+// state agree bitwise.
+template <int PREC, int Q, class LD, class SH>
+__device__ __forceinline__ auto set_moments(const LD& ld, const SH& sh, double K) {
   if constexpr (PREC == 2)
-    return moments_join<QH, V>(moments<QH, 1, V>(ld), sh, KH16);
+    return moments_shifted<Q>(ld, sh, K);
   else if constexpr (PREC == 1)
-    return moments_pairs<QH>(ld);
+    return moments_pairs<Q>(ld);
   else
-    return moments<QH, 0, V>(ld);
-}
-// The g moments in two parts: of the stored values, and (FP16S) joined with the
-// p* shifts.
-template <int PREC, int QG, class V, class LD>
-__device__ __forceinline__ Mom<V> g_moments_stored(const LD& ld) {
-  if constexpr (PREC == 1)
-    return moments_pairs<QG>(ld);
-  else
-    return moments<QG, PREC == 2, V>(ld);
-}
-template <int PREC, int QG, class V, class SH>
-__device__ __forceinline__ Mom<V> g_moments_shift(const Mom<V>& a, const SH& sh) {
-  if constexpr (PREC == 2)
-    return moments_join<QG, V>(a, sh, KG16);
-  else
-    return a;
+    return moments<Q, D1>(ld);
 }
 
 // ---------------------------------------------------------------------------
@@ -530,9 +506,32 @@ __device__ __forceinline__ Grad<V> phi_grad_flat(const PhiPlane<V>& o) {  // phi
   const V half = vbc<V>(0.5);
   return Grad<V>{half * o.gx, half * o.gy, vbc<V>(0.0), o.q};
 }
+// The same stencil over the D3Q27 (or D2Q9) weights by opposite pairs, in the
+// order of FP32 and FP16S (see collide_pairs).  phi_at(cx, cy, cz): phi^t at a
+// stencil neighbour.
+template <int QG, class PhiAt>
+__device__ __forceinline__ Grad<F1> phi_grad_pairs(const PhiAt& phi_at) {
+  typedef F1 V;
+  const V pc{phi_at(0, 0, 0)};
+  V gx = {}, gy = {}, gz = {}, lap = {};
+#pragma unroll
+  for (int i = 0; i < (QG - 1) / 2; ++i) {
+    const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
+    const V a{phi_at(cx, cy, cz)}, b{phi_at(-cx, -cy, -cz)};
+    const V w = vbc<V>(lq_w<QG>(i)), d = a - b;
+    const V t = (a - pc) + (b - pc);  // differences first: exact for nearby values
+    // (member 0 has every component of the lattice)
+    if (cx) gx = i ? vfma(cx > 0 ? w : -w, d, gx) : (cx > 0 ? w : -w) * d;
+    if (cy) gy = i ? vfma(cy > 0 ? w : -w, d, gy) : (cy > 0 ? w : -w) * d;
+    if (cz) gz = i ? vfma(cz > 0 ? w : -w, d, gz) : (cz > 0 ? w : -w) * d;
+    lap = i ? vfma(w, t, lap) : w * t;
+  }
+  const V three = vbc<V>(3.0);
+  return Grad<V>{gx * three, gy * three, gz * three, lap * vbc<V>(6.0)};
+}
 
 // ---------------------------------------------------------------------------
-// The step's parameters in the arithmetic type, formed once on the host.
+// The FP64 step's parameters, formed once on the host.
 template <class V>
 struct PhysV {
   V rho_l, drho, tau_l, dtau, beta4, mkappa, mdrho3, gx, gy, gz;
@@ -560,8 +559,8 @@ inline PhysV<V> phys_v(const Phys& p) {
   return q;
 }
 
-// The same without the combined factors, in the arithmetic type R (the FP32
-// step and the adjoint).
+// The same without the combined factors, in the arithmetic type R (the FP32 and
+// FP16S steps and the adjoint).
 template <typename R>
 struct PhysR {
   R rho_l, drho, tau_l, dtau, beta, kappa, inv_xi, omega_phi, gx, gy, gz;
@@ -588,24 +587,19 @@ inline PhysR<R> phys_r(const Phys& p) {
 template <int PREC>
 struct StepV {
   typedef F1 T;
-  typedef PhysV<F1> Par;
+  typedef PhysR<float> Par;
 };
 template <>
 struct StepV<0> {
   typedef D1 T;
   typedef PhysV<D1> Par;
 };
-template <>
-struct StepV<1> {
-  typedef F1 T;
-  typedef PhysR<float> Par;
-};
 template <int PREC>
 inline typename StepV<PREC>::Par step_par(const Phys& p) {
-  if constexpr (PREC == 1)
-    return phys_r<float>(p);
+  if constexpr (PREC == 0)
+    return phys_v<D1>(p);
   else
-    return phys_v<typename StepV<PREC>::T>(p);
+    return phys_r<float>(p);
 }
 
 // Emits the post-collision pairs of a quadratic polynomial of the velocity,
@@ -613,10 +607,9 @@ inline typename StepV<PREC>::Par step_par(const Phys& p) {
 // sharing the partial sums between directions: 21 additions for the even parts
 // and 10 for the odd ones of D3Q27 instead of 45 and 27.  put(i, oi, cx, cy,
 // cz, A, B): A for direction c (member i), B for -c (member oi).
-// F16: A = E + L, B = E - L (values divided by the weight).  Else the stored
-// value w (s + E +- L) with s the large part added last, one rounding at its
-// size.
-template <int Q, bool F16, class V, class PUT>
+// The stored value is w (s + E +- L) with s the large part added last, one
+// rounding at its size.
+template <int Q, class V, class PUT>
 __device__ __forceinline__ void emit_pairs(V s, V al, V bx, V by, V bz, V Gxx, V Gyy, V Gzz, V Gxy, V Gyz, V Gxz,
                                            const PUT& put) {
   const V Ex = al + Gxx, Ey = al + Gyy, Ez = al + Gzz;
@@ -650,16 +643,9 @@ __device__ __forceinline__ void emit_pairs(V s, V al, V bx, V by, V bz, V Gxx, V
       const V b2 = qy > 0 ? bxy : bxny;
       L = qz > 0 ? b2 + bz : b2 - bz;
     }
-    V A, B;  // of +q and -q
-    if constexpr (F16) {
-      A = E + L;
-      B = E - L;
-    } else {
-      const double w = lq_w<Q>(i);
-      const V e = vbc<V>(w) * E;
-      A = vfma(vbc<V>(w), s, vfma(vbc<V>(w), L, e));
-      B = vfma(vbc<V>(w), s, vfma(vbc<V>(-w), L, e));
-    }
+    const double w = lq_w<Q>(i);
+    const V e = vbc<V>(w) * E;
+    const V A = vfma(vbc<V>(w), s, vfma(vbc<V>(w), L, e)), B = vfma(vbc<V>(w), s, vfma(vbc<V>(-w), L, e));  // of +q and -q
     if (sgn > 0)
       put(i, Q - 1 - i, cx, cy, cz, A, B);
     else
@@ -667,23 +653,20 @@ __device__ __forceinline__ void emit_pairs(V s, V al, V bx, V by, V bz, V Gxx, V
   }
 }
 // the rest population of the same polynomial
-template <int Q, bool F16, class V>
+template <int Q, class V>
 __device__ __forceinline__ V emit_rest(V s, V al) {
-  if constexpr (F16) return al;
   const double w = lq_w<Q>((Q - 1) / 2);
   return vfma(vbc<V>(w), s, vbc<V>(w) * al);
 }
 
-// The collision of both sets (moments to post-collision populations) of FP64
-// and FP16S, shared by every stream-collide kernel.
+// The collision of both sets (moments to post-collision populations) of FP64,
+// shared by every stream-collide kernel.
 //   pc, gr: phi^t of the cell and its stencil; gm: the g moments;
 //   hmom(): the h moments, read when their turn comes;
-//   out.shift(pst): FP16S, stores P = fp16(p*) of the cell and returns it;
 //   out.grest(v), out.g_(i, oi, cx, cy, cz, A, B), out.hrest(v), out.h_(...).
-template <int PREC, int QH, class V, class HM, class OUT>
+template <int QH, class V, class HM, class OUT>
 __device__ __forceinline__ void collide(const PhysV<V>& ph, V pc, const Grad<V>& gr, const Mom<V>& gm, const HM& hmom,
                                         OUT& out) {
-  constexpr bool F16 = PREC == 2;
   constexpr int QG = qg_of<QH>();  // D2Q9 with the 2-D phase field, else D3Q27
   const V third = vbc<V>(1.0 / 3.0), one = vbc<V>(1.0), half = vbc<V>(0.5);
   const V pst = gm.s;
@@ -713,9 +696,7 @@ __device__ __forceinline__ void collide(const PhysV<V>& ph, V pc, const Grad<V>&
     uy = vfma(Fy, hr, gm.y);
     uz = vfma(Fz, hr, gm.z);
 
-    // ---- g post-collision coefficients and pair stores.  FP16S scales them
-    // by the format's power of two and stores deviations from P = fp16(p*).
-    constexpr double K = F16 ? KG16 : 1.0;
+    // ---- g post-collision coefficients and pair stores
     const V mx = -ux, my = -uy, mz = -uz;
     const V qx = mx * ux, qy = my * uy, qz = mz * uz;  // -u_a^2
     // deviatoric second moments, (3 P_aa - p*) / 3 with one rounding: p* (1/3)
@@ -724,52 +705,39 @@ __device__ __forceinline__ void collide(const PhysV<V>& ph, V pc, const Grad<V>&
     const V mp = -pst, three = vbc<V>(3.0);
     const V dxx = vfma(vfma(three, gm.xx, mp), third, qx), dyy = vfma(vfma(three, gm.yy, mp), third, qy);
     const V dzz = QG == 9 ? vbc<V>(0.0) : vfma(vfma(three, gm.zz, mp), third, qz);  // 2-D: the trace runs over x and y
-    const V a2 = vfma(vbc<V>(-4.5 * K), omega, vbc<V>(4.5 * K));
-    const V al = vfma(vbc<V>(1.5 * K), (qx + qy) + qz, (a2 * vbc<V>(-1.0 / 3.0)) * ((dxx + dyy) + dzz));
-    const V fr = vbc<V>(1.5 * K) * rinv, k3 = vbc<V>(3.0 * K);
+    const V a2 = vfma(vbc<V>(-4.5), omega, vbc<V>(4.5));
+    const V al = vfma(vbc<V>(1.5), (qx + qy) + qz, (a2 * vbc<V>(-1.0 / 3.0)) * ((dxx + dyy) + dzz));
+    const V fr = vbc<V>(1.5) * rinv, k3 = three;
     const V bx = vfma(fr, Fx, k3 * ux), by = vfma(fr, Fy, k3 * uy), bz = vfma(fr, Fz, k3 * uz);
-    const V k45 = vbc<V>(-4.5 * K), k9 = vbc<V>(-9.0 * K), a22 = a2 + a2;
+    const V k45 = vbc<V>(-4.5), k9 = vbc<V>(-9.0), a22 = a2 + a2;
     const V Gxx = vfma(k45, qx, a2 * dxx), Gyy = vfma(k45, qy, a2 * dyy), Gzz = vfma(k45, qz, a2 * dzz);
     const V qxy = mx * uy, qyz = my * uz, qxz = mx * uz;
     const V Gxy = vfma(k9, qxy, a22 * (gm.xy + qxy)), Gyz = vfma(k9, qyz, a22 * (gm.yz + qyz)),
             Gxz = vfma(k9, qxz, a22 * (gm.xz + qxz));
-    V e0 = al;
-    if constexpr (F16) e0 = vfma(vbc<V>(K), pst - out.shift(pst), al);
-    out.grest(emit_rest<QG, F16>(pst, e0));
-    emit_pairs<QG, F16>(pst, e0, bx, by, bz, Gxx, Gyy, Gzz, Gxy, Gyz, Gxz,
-                        [&](int i, int oi, int cx, int cy, int cz, V A, V B) { out.g_(i, oi, cx, cy, cz, A, B); });
+    out.grest(emit_rest<QG>(pst, al));
+    emit_pairs<QG>(pst, al, bx, by, bz, Gxx, Gyy, Gzz, Gxy, Gyz, Gxz,
+                   [&](int i, int oi, int cx, int cy, int cz, V A, V B) { out.g_(i, oi, cx, cy, cz, A, B); });
   }
 
   // ---- h post-collision coefficients and pair stores
   {
-    constexpr double K = F16 ? KH16 : 1.0;
     const Mom<V> h = hmom();
     const V gn = vsqrt(vfma(gr.z, gr.z, vfma(gr.y, gr.y, gr.x * gr.x)));
     // (1 - omega_phi / 2) theta / |grad phi|, theta = 4 phi (1 - phi) / xi
     const V tn = vdiv((ph.c4 * pc) * (one - pc), gn + vbc<V>(1e-6));
     // deviatoric second moments as (3 H_aa - phi) / 3 and the non-equilibrium
     // flux J - phi u, one rounding each
-    const V mphi = -h.s, three = vbc<V>(3.0), a2_3 = F16 ? vbc<V>(K) * ph.a2_3 : ph.a2_3;
-    const V Gxx = a2_3 * vfma(three, h.xx, mphi), Gyy = a2_3 * vfma(three, h.yy, mphi);
-    const V Gzz = QG == 9 ? vbc<V>(0.0) : a2_3 * vfma(three, h.zz, mphi);
+    const V mphi = -h.s, three = vbc<V>(3.0);
+    const V Gxx = ph.a2_3 * vfma(three, h.xx, mphi), Gyy = ph.a2_3 * vfma(three, h.yy, mphi);
+    const V Gzz = QG == 9 ? vbc<V>(0.0) : ph.a2_3 * vfma(three, h.zz, mphi);
     const V al = vbc<V>(-1.0 / 3.0) * ((Gxx + Gyy) + Gzz);
     const V p3 = three * h.s;
-    V bx = vfma(p3, ux, vfma(ph.a1, vfma(mphi, ux, h.x), tn * gr.x));
-    V by = vfma(p3, uy, vfma(ph.a1, vfma(mphi, uy, h.y), tn * gr.y));
-    V bz = vfma(p3, uz, vfma(ph.a1, vfma(mphi, uz, h.z), tn * gr.z));
-    V a2 = ph.a2;
-    V e0 = al;
-    if constexpr (F16) {
-      const V k = vbc<V>(K);
-      bx = k * bx;
-      by = k * by;
-      bz = k * bz;
-      a2 = k * a2;
-      e0 = vfma(k, h.s - pc, al);  // phi of the cell is the shift of everything it writes
-    }
-    out.hrest(emit_rest<QH, F16>(h.s, e0));
-    emit_pairs<QH, F16>(h.s, e0, bx, by, bz, Gxx, Gyy, Gzz, a2 * h.xy, a2 * h.yz, a2 * h.xz,
-                        [&](int i, int oi, int cx, int cy, int cz, V A, V B) { out.h_(i, oi, cx, cy, cz, A, B); });
+    const V bx = vfma(p3, ux, vfma(ph.a1, vfma(mphi, ux, h.x), tn * gr.x));
+    const V by = vfma(p3, uy, vfma(ph.a1, vfma(mphi, uy, h.y), tn * gr.y));
+    const V bz = vfma(p3, uz, vfma(ph.a1, vfma(mphi, uz, h.z), tn * gr.z));
+    out.hrest(emit_rest<QH>(h.s, al));
+    emit_pairs<QH>(h.s, al, bx, by, bz, Gxx, Gyy, Gzz, ph.a2 * h.xy, ph.a2 * h.yz, ph.a2 * h.xz,
+                   [&](int i, int oi, int cx, int cy, int cz, V A, V B) { out.h_(i, oi, cx, cy, cz, A, B); });
   }
 }
 
@@ -783,43 +751,31 @@ __device__ __forceinline__ F1 wsum(double w, F1 s, F1 r) {
   return vfma(F1{hi}, s, vfma(F1{lo}, s, F1{hi} * r));
 }
 
-// The collision of both sets in FP32, written around opposite-velocity pairs.
-// It keeps the operation order, each fused multiply-add included, that FP32 runs
-// have had throughout, so their results stay as they are: where the flow
-// amplifies FP32's rounding (the normal of a nearly uniform phi) another order
-// moves single cells by 1e-3 within 64 steps of a Taylor bubble, with no smaller
-// error against FP64.  The FP32 step is bound by memory, not by these operations.
-//   phi_at(cx, cy, cz): phi^t at a stencil neighbour; the rest as in collide().
-// FP32 and FP64 stores add the small terms first and the large part once.
-template <int QH, class PhiAt, class HM, class OUT>
-__device__ __forceinline__ void collide_pairs(const PhysR<float>& par, const PhiAt& phi_at, const Mom<F1>& gm, const HM& hmom,
-                                              OUT& out) {
+// The collision of both sets in FP32 and FP16S, written around opposite-velocity
+// pairs.  It keeps the operation order, each fused multiply-add included, that
+// these formats' runs have had throughout, so their results stay as they are:
+// where the flow amplifies FP32's rounding (the normal of a nearly uniform phi)
+// another order moves single cells by 1e-3 within 64 steps of a Taylor bubble, with
+// no smaller error against FP64; in FP16S it moves last bits in front of the
+// stochastic rounding, which then rounds other values up (the sums of FP64,
+// collide(), put FP16S fields 5e-4 to 1e-3 apart and 1-3 % further from FP64 on
+// impact, bubble and wave).
+//   Arguments as in collide(), gr from phi_grad_pairs();
+//   out.shift(pst): FP16S, stores P = fp16(p*) of the cell and returns it.
+// FP32 stores add the small terms first and the large part once.  FP16S stores
+// K (f / w - shift), K the format's power of two (folded into the coefficients,
+// which it scales exactly) and the shift the cell's own (P, phi): E +- L as is.
+template <int PREC, int QH, class HM, class OUT>
+__device__ __forceinline__ void collide_pairs(const PhysR<float>& par, F1 pc, const Grad<F1>& gr, const Mom<F1>& gm,
+                                              const HM& hmom, OUT& out) {
   typedef F1 V;
+  constexpr bool F16 = PREC == 2;
   constexpr int QG = qg_of<QH>();   // D2Q9 with the 2-D phase field, else D3Q27
   constexpr int GR = (QG - 1) / 2;  // rest index of g
-  const V third = vbc<V>(1.0 / 3.0), one = vbc<V>(1.0), half = vbc<V>(0.5), three = vbc<V>(3.0), k45 = vbc<V>(4.5),
-          zero = vbc<V>(0.0);
+  const V third = vbc<V>(1.0 / 3.0), one = vbc<V>(1.0), half = vbc<V>(0.5), three = vbc<V>(3.0), zero = vbc<V>(0.0);
   const V rho_l{par.rho_l}, drho{par.drho}, tau_l{par.tau_l}, dtau{par.dtau}, beta{par.beta}, kappa{par.kappa};
 
-  // ---- phi stencil over D3Q27 weights, by pairs
-  const V pc{phi_at(0, 0, 0)};
-  V gx = zero, gy = zero, gz = zero, lap = zero;
-#pragma unroll
-  for (int i = 0; i < GR; ++i) {
-    const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
-    const V a{phi_at(cx, cy, cz)}, b{phi_at(-cx, -cy, -cz)};
-    const V w = vbc<V>(lq_w<QG>(i)), d = a - b;
-    const V t = (a - pc) + (b - pc);  // differences first: exact for nearby values
-    // (member 0 has every component of the lattice)
-    if (cx) gx = i ? vfma(cx > 0 ? w : -w, d, gx) : (cx > 0 ? w : -w) * d;
-    if (cy) gy = i ? vfma(cy > 0 ? w : -w, d, gy) : (cy > 0 ? w : -w) * d;
-    if (cz) gz = i ? vfma(cz > 0 ? w : -w, d, gz) : (cz > 0 ? w : -w) * d;
-    lap = i ? vfma(w, t, lap) : w * t;
-  }
-  gx = gx * three;
-  gy = gy * three;
-  gz = gz * three;
-  lap = lap * vbc<V>(6.0);
+  const V gx = gr.x, gy = gr.y, gz = gr.z, lap = gr.lap;
 
   // ---- forces and velocity
   const V pst = gm.s;
@@ -844,28 +800,46 @@ __device__ __forceinline__ void collide_pairs(const PhysR<float>& par, const Phi
 
   // ---- g post-collision coefficients and pair stores
   {
-    const V x2 = ux * ux, y2 = uy * uy, z2 = uz * uz;
-    const V uu = (x2 + y2) + z2;
-    const V a2 = (one - omega) * k45;
-    // deviatoric second moments, (3 P_aa - p*) / 3 with one rounding: p* (1/3)
-    // would carry the rounded constant 1/3, a bias of 3e-8 p* that repeats
-    // every step
-    const V dxx = vfma(vfma(three, gm.xx, -pst), third, -x2), dyy = vfma(vfma(three, gm.yy, -pst), third, -y2);
-    const V dzz = QG == 9 ? zero : vfma(vfma(three, gm.zz, -pst), third, -z2);  // 2-D: the trace runs over x and y
-    const V als = vfma(vbc<V>(-1.5), uu, -((a2 * ((dxx + dyy) + dzz)) * third));
-    const V fr = vdiv(vbc<V>(1.5), rho);
-    const V bx = vfma(fr, Fx, three * ux), by = vfma(fr, Fy, three * uy), bz = vfma(fr, Fz, three * uz);
+    constexpr double K = F16 ? KG16 : 1.0;
+    const V y2 = uy * uy;
+    V dxx, dyy, dzz, uu;
+    if constexpr (F16) {
+      uu = vfma(uz, uz, vfma(ux, ux, y2));
+      dxx = vfma(-ux, ux, gm.xx - p3);
+      dyy = (gm.yy - p3) - y2;
+      dzz = vfma(-uz, uz, gm.zz - p3);
+    } else {
+      // deviatoric second moments, (3 P_aa - p*) / 3 with one rounding: p* (1/3)
+      // would carry the rounded constant 1/3, a bias of 3e-8 p* that repeats
+      // every step
+      const V x2 = ux * ux, z2 = uz * uz;
+      uu = (x2 + y2) + z2;
+      dxx = vfma(vfma(three, gm.xx, -pst), third, -x2);
+      dyy = vfma(vfma(three, gm.yy, -pst), third, -y2);
+      dzz = vfma(vfma(three, gm.zz, -pst), third, -z2);
+    }
+    if (QG == 9) dzz = zero;  // 2-D: the trace runs over x and y
+    const V a2 = (one - omega) * vbc<V>(4.5 * K), k45 = vbc<V>(4.5 * K), k3 = vbc<V>(3.0 * K);
+    const V tr = a2 * ((dxx + dyy) + dzz);
+    V als;  // alpha less the large part
+    if constexpr (F16)
+      als = vfma(-tr, third, vfma(vbc<V>(-1.5 * K), uu, vbc<V>(K) * (pst - V{out.shift(pst.v)})));
+    else
+      als = vfma(vbc<V>(-1.5), uu, -(tr * third));
+    const V fr = vdiv(vbc<V>(1.5 * K), rho);
+    const V bx = vfma(fr, Fx, k3 * ux), by = vfma(fr, Fy, k3 * uy), bz = vfma(fr, Fz, k3 * uz);
     const V tx = k45 * ux, ty = k45 * uy, tz = k45 * uz;
     const V Gxx = vfma(tx, ux, a2 * dxx), Gyy = vfma(ty, uy, a2 * dyy), Gzz = vfma(tz, uz, a2 * dzz);
     const V two = vbc<V>(2.0);
     const V Gxy = two * vfma(tx, uy, a2 * vfma(-ux, uy, gm.xy));
     const V Gyz = two * vfma(ty, uz, a2 * vfma(-uy, uz, gm.yz));
     const V Gxz = two * vfma(tx, uz, a2 * vfma(-ux, uz, gm.xz));
-    out.grest(wsum(lq_w<QG>(GR), pst, als));
+    out.grest(F16 ? als : wsum(lq_w<QG>(GR), pst, als));
 #pragma unroll
     for (int i = 0; i < GR; ++i) {
       const int cx = q27_cx(lq_to27<QG>(i)), cy = q27_cy(lq_to27<QG>(i)), cz = q27_cz(lq_to27<QG>(i));
       V E = cx ? Gxx : (cy ? Gyy : Gzz);
+      if (F16) E = als + E;
       if (cx && cy) E = E + Gyy;
       if ((cx || cy) && cz) E = E + Gzz;
       if (cx && cy) E = E + ((cx * cy > 0) ? Gxy : -Gxy);
@@ -874,34 +848,56 @@ __device__ __forceinline__ void collide_pairs(const PhysR<float>& par, const Phi
       V L = cx ? (cx > 0 ? bx : -bx) : (cy ? (cy > 0 ? by : -by) : (cz > 0 ? bz : -bz));
       if (cx && cy) L = L + (cy > 0 ? by : -by);
       if ((cx || cy) && cz) L = L + (cz > 0 ? bz : -bz);
-      out.g_(i, QG - 1 - i, cx, cy, cz, wsum(lq_w<QG>(i), pst, als + (E + L)), wsum(lq_w<QG>(i), pst, als + (E - L)));
+      if constexpr (F16)
+        out.g_(i, QG - 1 - i, cx, cy, cz, E + L, E - L);
+      else
+        out.g_(i, QG - 1 - i, cx, cy, cz, wsum(lq_w<QG>(i), pst, als + (E + L)), wsum(lq_w<QG>(i), pst, als + (E - L)));
     }
   }
 
   // ---- h post-collision coefficients and pair stores
   {
+    constexpr double K = F16 ? KH16 : 1.0;
     const Mom<F1> h = hmom();
     const V phl = h.s, omp{par.omega_phi};
     const V gn = vsqrt(vfma(gz, gz, vfma(gy, gy, gx * gx)));
     const V theta = ((vbc<V>(4.0) * pc) * (one - pc)) * V{par.inv_xi};
-    const V tn = vdiv(theta, gn + vbc<V>(1e-6)) * (one - half * omp);  // (1 - omega_phi/2) theta / |grad phi|
-    const V a1 = (one - omp) * three, a2 = (one - omp) * k45;
-    // deviatoric second moments as (3 H_aa - phi) / 3 and the non-equilibrium
-    // flux J - phi u, one rounding each
-    const V dxx = vfma(three, h.xx, -phl) * third, dyy = vfma(three, h.yy, -phl) * third;
-    const V dzz = QG == 9 ? zero : vfma(three, h.zz, -phl) * third;
-    const V als = ((-a2) * ((dxx + dyy) + dzz)) * third;
-    const V p3 = three * phl;
+    // (1 - omega_phi/2) theta / |grad phi|
+    const V tn = vdiv(theta, gn + vbc<V>(1e-6)) * (vbc<V>(K) * (one - half * omp));
+    const V a1 = (one - omp) * vbc<V>(3.0 * K), a2 = (one - omp) * vbc<V>(4.5 * K);
+    V dxx, dyy, dzz;
+    if constexpr (F16) {
+      dxx = vfma(-phl, third, h.xx);
+      dyy = vfma(-phl, third, h.yy);
+      dzz = vfma(-phl, third, h.zz);
+    } else {
+      // deviatoric second moments as (3 H_aa - phi) / 3, one rounding each
+      dxx = vfma(three, h.xx, -phl) * third;
+      dyy = vfma(three, h.yy, -phl) * third;
+      dzz = vfma(three, h.zz, -phl) * third;
+    }
+    if (QG == 9) dzz = zero;
+    V als;
+    if constexpr (F16)  // phi of the cell is the shift of everything it writes
+      als = vfma(-(a2 * ((dxx + dyy) + dzz)), third, vbc<V>(K) * (phl - pc));
+    else
+      als = ((-a2) * ((dxx + dyy) + dzz)) * third;
+    // (the non-equilibrium flux J - phi u with one rounding)
+    const V p3 = vbc<V>(3.0 * K) * phl;
     const V bx = vfma(tn, gx, vfma(p3, ux, a1 * vfma(-phl, ux, h.x)));
     const V by = vfma(tn, gy, vfma(p3, uy, a1 * vfma(-phl, uy, h.y)));
     const V bz = vfma(tn, gz, vfma(p3, uz, a1 * vfma(-phl, uz, h.z)));
     const V a22 = vbc<V>(2.0) * a2;
     const V Hxx = a2 * dxx, Hyy = a2 * dyy, Hzz = a2 * dzz;
-    out.hrest(wsum(hq_w<QH>(hq_rest<QH>()), phl, als));
+    out.hrest(F16 ? als : wsum(hq_w<QH>(hq_rest<QH>()), phl, als));
 #pragma unroll
     for (int k = 0; k < hq_rest<QH>(); ++k) {
       const int cx = hq_cx<QH>(k), cy = hq_cy<QH>(k), cz = hq_cz<QH>(k);
-      V E = cx ? Hxx : (cy ? Hyy : Hzz);
+      V E;
+      if constexpr (F16)
+        E = vfma(a2, cx ? dxx : (cy ? dyy : dzz), als);
+      else
+        E = cx ? Hxx : (cy ? Hyy : Hzz);
       if (cx && cy) E = vfma(a2, dyy, E);
       if ((cx || cy) && cz) E = vfma(a2, dzz, E);
       if (cx && cy) E = vfma((cx * cy > 0) ? a22 : -a22, h.xy, E);
@@ -910,7 +906,10 @@ __device__ __forceinline__ void collide_pairs(const PhysR<float>& par, const Phi
       V L = cx ? (cx > 0 ? bx : -bx) : (cy ? (cy > 0 ? by : -by) : (cz > 0 ? bz : -bz));
       if (cx && cy) L = L + (cy > 0 ? by : -by);
       if ((cx || cy) && cz) L = L + (cz > 0 ? bz : -bz);
-      out.h_(k, QH - 1 - k, cx, cy, cz, wsum(hq_w<QH>(k), phl, als + (E + L)), wsum(hq_w<QH>(k), phl, als + (E - L)));
+      if constexpr (F16)
+        out.h_(k, QH - 1 - k, cx, cy, cz, E + L, E - L);
+      else
+        out.h_(k, QH - 1 - k, cx, cy, cz, wsum(hq_w<QH>(k), phl, als + (E + L)), wsum(hq_w<QH>(k), phl, als + (E - L)));
     }
   }
 }
@@ -958,9 +957,9 @@ __device__ __forceinline__ Mom<typename StepV<PREC>::T> h_moments_cell(
     unsigned N, const typename Store<PREC>::S* h, const typename Store<PREC>::PhiT* __restrict__ shift, unsigned cell,
     const CellOff& o) {
   typedef typename StepV<PREC>::T V;
-  return h_moments<PREC, QH, V>(
+  return set_moments<PREC, QH>(
       [&](int cx, int cy, int cz) { return V{load_dir<PREC, QH, READ_ODD>(h, N, cell, o, cx, cy, cz)}; },
-      [&](int cx, int cy, int cz) { return V{(typename V::R)__ldg(shift + writer(cell, o, cx, cy, cz))}; });
+      [&](int cx, int cy, int cz) { return V{(typename V::R)__ldg(shift + writer(cell, o, cx, cy, cz))}; }, KH16);
 }
 
 // Destination of one cell's collision: the pairs go to (h, g) in the layout
@@ -973,10 +972,10 @@ struct CellOut {
   const CellOff& o;
   __half* pg_out;
   Dither dith;
-  __device__ __forceinline__ V shift(V pst) {
-    const __half q = __float2half_rn((float)pst.v);
+  __device__ __forceinline__ float shift(float pst) {
+    const __half q = __float2half_rn(pst);
     pg_out[cell] = q;
-    return V{(typename V::R)__half2float(q)};
+    return __half2float(q);
   }
   __device__ __forceinline__ void grest(V v) { g[(unsigned)((qg_of<QH>() - 1) / 2) * N + cell] = pack_sr<PREC>(v.v, dith); }
   __device__ __forceinline__ void hrest(V v) { h[(unsigned)hq_rest<QH>() * N + cell] = pack_sr<PREC>(v.v, dith); }
@@ -1004,19 +1003,18 @@ __device__ __forceinline__ void step_cell(const Geo32& geo, const typename StepV
   CellOff o;
   cell_off(geo, cell, o);
   auto at = [&](int cx, int cy, int cz) { return (R)__ldg(phi + cell + o.soff(cx, cy, cz)); };
-  const Mom<V> gm = g_moments_shift<PREC, QG, V>(
-      g_moments_stored<PREC, QG, V>(
-          [&](int cx, int cy, int cz) { return V{load_dir<PREC, QG, ODD>(g, geo.N, cell, o, cx, cy, cz)}; }),
-      [&](int cx, int cy, int cz) { return V{(R)__half2float(__ldg(pg_in + writer(cell, o, cx, cy, cz)))}; });
+  const Mom<V> gm = set_moments<PREC, QG>(
+      [&](int cx, int cy, int cz) { return V{load_dir<PREC, QG, ODD>(g, geo.N, cell, o, cx, cy, cz)}; },
+      [&](int cx, int cy, int cz) { return V{(R)__half2float(__ldg(pg_in + writer(cell, o, cx, cy, cz)))}; }, KG16);
   CellOut<PREC, QH, ODD> out{h, g, geo.N, cell, o, pg_out, Dither{PREC == 2 ? hash32(cell * 0x9E3779B1u + seed) : 0u}};
   auto hm = [&] { return h_moments_cell<PREC, QH, ODD>(geo.N, h, shift, cell, o); };
-  if constexpr (PREC == 1) {
-    collide_pairs<QH>(ph, at, gm, hm, out);
+  if constexpr (PREC != 0) {
+    collide_pairs<PREC, QH>(ph, F1{at(0, 0, 0)}, phi_grad_pairs<QG>(at), gm, hm, out);
   } else {
     auto plane = [&](int cz) { return phi_plane<V>([&](int cx, int cy) { return V{at(cx, cy, cz)}; }); };
     const PhiPlane<V> p0 = plane(0);
     const Grad<V> gr = QG == 9 ? phi_grad_flat(p0) : phi_grad(plane(-1), p0, plane(1));
-    collide<PREC, QH, V>(ph, p0.c, gr, gm, hm, out);
+    collide<QH, V>(ph, p0.c, gr, gm, hm, out);
   }
 }
 
@@ -1141,14 +1139,14 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
   constexpr int NRING = 2 * (PW + PH) - 4;
   constexpr bool F16 = PREC == 2;
   constexpr int QG = qg_of<QH>();
-  // phi planes.  MARCH: the one being filled and the one being read, whose
+  // phi planes.  MARCH (FP64): the one being filled and the one being read, whose
   // in-plane stencil part is kept in registers (two slots, one barrier per
   // plane: a slot is refilled only after the barrier that follows its last
-  // read).  FP32, and solid cells, whose stencil reads depend on the reading
-  // cell: all three planes of the stencil and the one being filled (FP64: three
-  // slots, within 48 KB of static shared memory, and a second barrier).  The p*
-  // shifts are read for three planes as well.  The h moments are per thread.
-  constexpr bool MARCH = PREC != 1 && !SOLID;
+  // read).  FP32 and FP16S, and solid cells, whose stencil reads depend on the
+  // reading cell: all three planes of the stencil and the one being filled (FP64:
+  // three slots, within 48 KB of static shared memory, and a second barrier).  The
+  // p* shifts are read for three planes as well.  The h moments are per thread.
+  constexpr bool MARCH = PREC == 0 && !SOLID;
   constexpr int NS = FLAT ? 1 : (MARCH ? 2 : (sizeof(R) == 8 ? 3 : 4));
   constexpr int NSP = FLAT ? 1 : 4;
   // FP32 gathers the g populations of the plane about to collide before the next
@@ -1211,26 +1209,33 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
     if (F16) o = off_xyz(geo, qx, qy, zq, SOLID ? __ldg(links + c) : 0u);
     return (PhiT)h_moments_cell<PREC, QH, 0>(N, hA, phi_shift, c, o).s.v;
   };
+  // ring cell r of a plane: its place in the ring, its column
+  struct RingCell {
+    int at;
+    unsigned x, y;
+  };
+  auto ring_cell = [&](int r) {
+    int i, j;
+    frame_pos(r, PW, PH, i, j);
+    return RingCell{j * PW + i, (unsigned)wrap_or_clamp(x0 - 1 + i, (int)geo.nx, geo.wall[0]),
+                    (unsigned)wrap_or_clamp(y0 - 1 + j, (int)geo.ny, geo.wall[1])};
+  };
+  // FP16S finds its ring cell once (bubble 128x384x128: 410 -> 398 us per step; FP64
+  // is indifferent, and FP32 planes lose, 5.65 -> 5.84 us on 200x400).
+  static_assert(!F16 || NRING <= NT, "one ring cell per thread");
+  const RingCell own_ring = ring_cell(min(tid, NRING - 1));
   // phi of plane zp over the tile (with the h moments of the own cells) and its ring
   auto fill = [&](int zp, int slot, int pslot, int mslot) {
     const unsigned zq = (unsigned)wrap_or_clamp(zp, (int)geo.nz, geo.wall[2]);
     const unsigned c = xq + geo.nx * (yq + geo.ny * zq);
     CellOff o;
     if (F16) o = off_xyz(geo, xq, yq, zq, SOLID ? __ldg(links + c) : 0u);
-    // ring cell r: its place in the ring, phi and, FP16S, p* shift
-    auto ring_cell = [&](int r, int& at, PhiT& v, float& pv) {
-      int ri, rj;
-      frame_pos(r, PW, PH, ri, rj);
-      const unsigned rx = (unsigned)wrap_or_clamp(x0 - 1 + ri, (int)geo.nx, geo.wall[0]);
-      const unsigned ry = (unsigned)wrap_or_clamp(y0 - 1 + rj, (int)geo.ny, geo.wall[1]);
-      at = rj * PW + ri;
-      v = phi_at(rx, ry, zq);
-      if constexpr (F16) pv = ld_pshift(pg_in, rx + geo.nx * (ry + geo.ny * zq));
-    };
-    int rat = 0;
+    RingCell rc = {};
     PhiT rv = 0;
-    float rp = 0;
-    if constexpr (RING1ST) ring_cell(NRING < NT ? min(tid, NRING - 1) : tid, rat, rv, rp);
+    if constexpr (RING1ST) {
+      rc = ring_cell(min(tid, NRING - 1));
+      rv = phi_at(rc.x, rc.y, zq);
+    }
     if constexpr (TM != 0) ok = mbar_wait(mbar, phase_h++ & 1) && ok;
     if (PREC == 0 && !FLAT && (zp < z0 || zp >= z1)) {
       // FP64, the planes beside the chunk: their cells collide in other blocks, so
@@ -1240,13 +1245,13 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
       // lose 3 % by the second code site.
       ring[slot][i0] = phi_at(xq, yq, zq);
     } else {
-      const Mom<V> m = h_moments<PREC, QH, V>(
+      const Mom<V> m = set_moments<PREC, QH>(
           [&](int cx, int cy, int cz) {
             const unsigned i = (unsigned)lq_index<QH>(cx, cy, cz);
             if constexpr (TM != 0) return V{raw<PREC>(sH[i * NT + tid])};
             return V{raw<PREC>(hA[i * N + c])};
           },
-          [&](int cx, int cy, int cz) { return V{(R)__ldg(phi_shift + writer(c, o, cx, cy, cz))}; });
+          [&](int cx, int cy, int cz) { return V{(R)__ldg(phi_shift + writer(c, o, cx, cy, cz))}; }, KH16);
       // (tile positions outside the lattice serve as ring cells; the copy does not hold them)
       ring[slot][i0] = TM && !active ? phi_at(xq, yq, zq) : (PhiT)m.s.v;
       V* hm = &hmom[mslot][tid];
@@ -1262,14 +1267,13 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
       hm[9 * NT] = m.xz;
     }
     if constexpr (F16) pring[pslot][i0] = ld_pshift(pg_in, c);
-    if (RING1ST && tid < NRING) ring[slot][rat] = rv;
+    if (RING1ST && tid < NRING) ring[slot][rc.at] = rv;
 #pragma unroll
     for (int r0 = RING1ST ? NT : 0; r0 < NRING; r0 += NT) {
-      const int r = r0 + tid;
-      if (r < NRING) {
-        ring_cell(r, rat, rv, rp);
-        ring[slot][rat] = rv;
-        if constexpr (F16) pring[pslot][rat] = rp;
+      if (r0 + tid < NRING) {
+        const RingCell q = F16 ? own_ring : ring_cell(r0 + tid);
+        ring[slot][q.at] = phi_at(q.x, q.y, zq);
+        if constexpr (F16) pring[pslot][q.at] = ld_pshift(pg_in, q.x + geo.nx * (q.y + geo.ny * zq));
       }
     }
   };
@@ -1278,25 +1282,30 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
     return phi_plane<V>([&](int cx, int cy) { return V{(R)ring[slot][i0 + cy * PW + cx]}; });
   };
 
-  // g moments of the own cell of plane z (plane count b): the stored values,
-  // then the p* shifts
+  // g moments of the own cell of plane z (plane count b)
   unsigned cell = 0;
   CellOff o;
   Mom<V> gm = {};
-  auto gather_g = [&] {
-    gm = g_moments_stored<PREC, QG, V>([&](int cx, int cy, int cz) {
-      const unsigned i = (unsigned)lq_index<QG>(cx, cy, cz);
-      if constexpr (TM != 0) return V{raw<PREC>(sG[i * NT + tid])};
-      return V{raw<PREC>(gA[i * N + cell])};
-    });
-  };
-  auto shift_g = [&](int b) {
-    gm = g_moments_shift<PREC, QG, V>(gm, [&](int cx, int cy, int cz) {
-      // p* of the writer x - c, or of the cell itself after a bounce-back
-      const float* p0 = pring[FLAT ? 0 : b % NSP];
-      const float* pz = FLAT ? p0 : pring[(b - cz) % NSP];
-      return V{o.valid(-cx, -cy, -cz) ? (R)pz[i0 - cy * PW - cx] : (R)p0[i0]};
-    });
+  auto gather_g = [&](int b) {
+    gm = set_moments<PREC, QG>(
+        [&](int cx, int cy, int cz) {
+          const unsigned i = (unsigned)lq_index<QG>(cx, cy, cz);
+          if constexpr (TM != 0) return V{raw<PREC>(sG[i * NT + tid])};
+          return V{raw<PREC>(gA[i * N + cell])};
+        },
+        [&](int cx, int cy, int cz) {
+          // p* of the writer x - c, or of the cell itself after a bounce-back
+          // (solid cells: one index from the start of the planes; Taylor tube 62x600x62
+          // 206 -> 199 us per step, but bubble 128x384x128 without solids 398 -> 419)
+          if constexpr (SOLID && F16) {
+            const int own = (FLAT ? 0 : (b & 3) * PS) + i0, at = (FLAT ? 0 : ((b - cz) & 3) * PS) + i0 - cy * PW - cx;
+            return V{(&pring[0][0])[o.valid(-cx, -cy, -cz) ? at : own]};
+          }
+          const float* p0 = pring[FLAT ? 0 : b % NSP];
+          const float* pz = FLAT ? p0 : pring[(b - cz) % NSP];
+          return V{o.valid(-cx, -cy, -cz) ? (R)pz[i0 - cy * PW - cx] : (R)p0[i0]};
+        },
+        KG16);
   };
 
   // Planes z0 - 1 .. z1 are filled in turn; once plane z + 1 is, plane z
@@ -1309,7 +1318,7 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
     const int bp = zp - (z0 - 1), b = bp - 1;  // plane counts from z0 - 1
     cell = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)z);
     if (TM && z >= z0) ok = mbar_wait(mbar + 8, phase_g++ & 1) && ok;
-    if (EARLY && z >= z0 && (TM || active)) gather_g();
+    if (EARLY && z >= z0 && (TM || active)) gather_g(b);
     fill(FLAT ? 0 : zp, FLAT ? 0 : bp % NS, FLAT ? 0 : bp % NSP, FLAT ? 0 : bp & 1);
     if constexpr (TM != 0) {
       if (!__syncthreads_and(ok)) {
@@ -1342,30 +1351,30 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
         if (blk & link_bit(cx, cy, cz)) return (R)at0[i0];
         return (R)(FLAT ? at0 : ring[(b + cz) % NS])[i0 + cy * PW + cx];
       };
-      // solid cells: the stencil before g, whose moments then hold no registers
-      // meanwhile (FP16S Taylor tube 62x600x62: 217 -> 206 us per step)
-      V sc = {};
-      Grad<V> sgr = {};
-      if constexpr (PREC != 1 && !MARCH) {
+      // FP64 and FP16S: the stencil before g, whose moments then hold no registers
+      // meanwhile
+      if (PREC == 1 && !EARLY) gather_g(b);
+      const V pc = MARCH ? po.c : V{(R)at0[i0]};
+      Grad<V> gr;
+      if constexpr (PREC != 0) {
+        gr = phi_grad_pairs<QG>(at);
+      } else if constexpr (MARCH) {
+        gr = FLAT ? phi_grad_flat(po) : phi_grad(pm, po, pp);
+      } else {
         auto splane = [&](int cz) { return phi_plane<V>([&](int cx, int cy) { return V{at(cx, cy, cz)}; }); };
         const PhiPlane<V> p0 = splane(0);
-        sc = p0.c;
-        sgr = QG == 9 ? phi_grad_flat(p0) : phi_grad(splane(-1), p0, splane(1));
+        gr = QG == 9 ? phi_grad_flat(p0) : phi_grad(splane(-1), p0, splane(1));
       }
-      if (!EARLY) gather_g();
-      shift_g(b);
+      if (PREC != 1) gather_g(b);
       CellOut<PREC, QH, 1> out{hB, gB, N, cell, o, pg_out, Dither{F16 ? hash32(cell * 0x9E3779B1u + seed) : 0u}};
       const V* hp = &hmom[FLAT ? 0 : b & 1][tid];
       auto hm = [&] {
         return Mom<V>{hp[0], hp[NT], hp[2 * NT], hp[3 * NT], hp[4 * NT], hp[5 * NT], hp[6 * NT], hp[7 * NT], hp[8 * NT], hp[9 * NT]};
       };
-      if constexpr (PREC == 1) {
-        collide_pairs<QH>(ph, at, gm, hm, out);
-      } else if constexpr (MARCH) {
-        collide<PREC, QH, V>(ph, po.c, FLAT ? phi_grad_flat(po) : phi_grad(pm, po, pp), gm, hm, out);
-      } else {
-        collide<PREC, QH, V>(ph, sc, sgr, gm, hm, out);
-      }
+      if constexpr (PREC != 0)
+        collide_pairs<PREC, QH>(ph, pc, gr, gm, hm, out);
+      else
+        collide<QH, V>(ph, pc, gr, gm, hm, out);
     }
     if (!FLAT) {
       pm = po;
