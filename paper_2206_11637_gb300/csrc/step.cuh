@@ -1029,7 +1029,7 @@ __device__ __forceinline__ CellOff off_xyz(const Geo32& geo, unsigned x, unsigne
 // TM: the tile's own populations come by tensor copies into dynamic shared
 // memory, one box of every member of h and of g per plane, issued as soon as the
 // plane before is read; `mbar` holds the two barriers (h, g).  Returns false if
-// a copy did not arrive.
+// a copy did not arrive within its wait's limit.
 template <int PREC, int QH, int TY, int FLAT, int SOLID, int TX = ZM_TX, int TM = 0>
 __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<PREC>::Par& ph,
                                         const typename Store<PREC>::S* __restrict__ hA,
@@ -1097,18 +1097,18 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
   extern __shared__ __align__(128) unsigned char dyn[];
   S* sG = (S*)dyn;
   S* sH = sG + QG * NT;
-  unsigned phase_h = 0, phase_g = 0;
+  CopyGate gate_h{mbar}, gate_g{mbar + 8};
   bool ok = true;
   auto issue_h = [&](int zp) {
     if (tid == 0) {
-      mbar_expect(mbar, QH * NT * sizeof(S));
-      tma4(smem_u32(sH), &maps->h, x0, y0, wrap_or_clamp(zp, (int)geo.nz, geo.wall[2]), 0, mbar);
+      mbar_expect(gate_h.bar, QH * NT * sizeof(S));
+      tma4(smem_u32(sH), &maps->h, x0, y0, wrap_or_clamp(zp, (int)geo.nz, geo.wall[2]), 0, gate_h.bar);
     }
   };
   auto issue_g = [&](int z) {
     if (tid == 0) {
-      mbar_expect(mbar + 8, QG * NT * sizeof(S));
-      tma4(smem_u32(sG), &maps->g, x0, y0, z, 0, mbar + 8);
+      mbar_expect(gate_g.bar, QG * NT * sizeof(S));
+      tma4(smem_u32(sG), &maps->g, x0, y0, z, 0, gate_g.bar);
     }
   };
 
@@ -1146,7 +1146,7 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
       rc = ring_cell(min(tid, NRING - 1));
       rv = phi_at(rc.x, rc.y, zq);
     }
-    if constexpr (TM != 0) ok = mbar_wait(mbar, phase_h++ & 1) && ok;
+    if constexpr (TM != 0) ok = gate_h.wait() && ok;
     if (PREC == 0 && !FLAT && (zp < z0 || zp >= z1)) {
       // FP64, the planes beside the chunk: their cells collide in other blocks, so
       // phi alone (14 additions instead of 39): drop 32^3, one plane per chunk,
@@ -1227,14 +1227,14 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
     const int z = FLAT ? zp : zp - 1;
     const int bp = zp - (z0 - 1), b = bp - 1;  // plane counts from z0 - 1
     cell = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)z);
-    if (TM && z >= z0) ok = mbar_wait(mbar + 8, phase_g++ & 1) && ok;
+    if (TM && z >= z0) ok = gate_g.wait() && ok;
     if (EARLY && z >= z0 && (TM || active)) gather_g(b);
     fill(FLAT ? 0 : zp, FLAT ? 0 : bp % NS, FLAT ? 0 : bp % NSP, FLAT ? 0 : bp & 1);
     if constexpr (TM != 0) {
       if (!__syncthreads_and(ok)) {
-        // give the copies in flight another bounded wait before the block's memory goes
-        mbar_wait(mbar, phase_h & 1);
-        mbar_wait(mbar + 8, phase_g & 1);
+        // (every copy issued so far has been waited for)
+        gate_h.drain();
+        gate_g.drain();
         return false;
       }
       if (zp < z1) issue_h(zp + 1);
@@ -1316,7 +1316,10 @@ __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
 
 // The same with the populations read by tensor copies (3-D lattices without
 // solid cells whose rows are whole 16-byte units), in tiles of TX x TY.  err: set
-// when a copy did not arrive.
+// when a copy did not arrive; the state is lost then, and blocks that find it set
+// return at once, so that later waves, steps and graph replays do not each wait for
+// their copies' limit.  (Read before the wait for the previous step, whose time
+// hides it: bubble 128x384x128 363.6 us per step without, 364.2 with.)
 template <int PREC, int QH, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
     k_step_tma(const __grid_constant__ StepMaps maps, Geo32 geo, typename StepV<PREC>::Par ph,
@@ -1331,8 +1334,9 @@ __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
     mbar_init(bar);
     mbar_init(bar + 8);
   }
-  __syncthreads();
+  const int lost = __syncthreads_or(*err);
   if (PFL_ZM_PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (lost) return;
   if (PREC == 2 && tclock) seed = step_seed_of(*tclock + (unsigned long long)tofs);
   if (!zm_tile<PREC, QH, TY, 0, 0, TX, 1>(geo, ph, hA, gA, hB, gB, phi_shift, phi_out, zc, seed, nullptr, pg_in, pg_out,
                                           blockIdx.x, blockIdx.y, blockIdx.z, &maps, bar) &&
