@@ -52,7 +52,7 @@ pfl_status cuda_fail(cudaError_t e, const char* what) {
 
 
 struct Layout {
-  size_t h, g, h2, g2, phi[2], pg[2], links, stage, red, clock, total;
+  size_t h, g, h2, g2, phi[2], pg[2], links, stage, red, clock, err, total;
 };
 
 Layout layout_of(const pfl_params* p) {
@@ -88,7 +88,8 @@ Layout layout_of(const pfl_params* p) {
   L.red = off;  // phi partials (9 per block), results, flow-speed partials (1 per block), result
   off = align256(off + (DIAG_BLOCKS * 10 + 32) * sizeof(double));
   L.clock = off;  // step count read by graph-replayed steps
-  off = align256(off + sizeof(unsigned long long));
+  L.err = off + 128;  // set by the fused step when a tensor copy did not arrive (in the same 256 bytes)
+  off = align256(off + 128 + sizeof(int));
   L.total = off;
   return L;
 }
@@ -133,20 +134,32 @@ struct pfl_ctx {
   long long cap_t0;         // step count when the capture began
   long long clock_t;        // step count the device clock holds (-1: unknown)
   // fused step with its loads by tensor copies: tile shape (index into
-  // TMA_TILES, -1: not used), maps of the two array pairs, and the host word a
-  // kernel reports to when a copy did not arrive
+  // TMA_TILES, -1: not used) and maps of the two array pairs
   int tma;
   StepMaps maps[2];
   EncodeTiled encode;
-  int* err;
   bool wide;     // fused step without copies in tiles of WIDE_TX x WIDE_TY
 };
 
 namespace {
 
-pfl_status check_err(const pfl_ctx* c) {
-  if (c->err && *(volatile int*)c->err)
-    return fail(PFL_ERR_CUDA, "a copy of the fused step did not arrive; the state is not valid");
+volatile int* err_of(const pfl_ctx* c) { return (volatile int*)(c->ws + c->L.err); }
+
+// Ends the calls that read the state out: reports a tensor copy that did not
+// arrive in the steps before.
+pfl_status check_copies(const pfl_ctx* c) {
+  if (c->tma < 0) return PFL_OK;
+  int lost = 0;
+  CUDA_TRY(cudaMemcpyAsync(&lost, (const void*)err_of(c), sizeof lost, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(cudaStreamSynchronize(c->stream));
+  if (lost)
+    return fail(PFL_ERR_CUDA, "a copy of the fused step did not arrive; the state is lost (pfl_load or pfl_set_populations replaces it)");
+  return PFL_OK;
+}
+
+// For a state that is replaced as a whole.
+pfl_status clear_copies(const pfl_ctx* c) {
+  if (c->tma >= 0) CUDA_TRY(cudaMemsetAsync((void*)err_of(c), 0, sizeof(int), c->stream));
   return PFL_OK;
 }
 
@@ -408,7 +421,7 @@ void step_only(pfl_ctx* c) {
       if constexpr (has_tma<PREC, QH>())
         tma_shape<PREC, QH>(c->tma, [&](auto k) {
           k.launch(c, cfg, c->maps[c->ab], c->g32, ph1, ha, ga, hnext<PREC>(c), gnext<PREC>(c), shift, phicur<PREC>(c), c->zc,
-                   step_seed(c), tclock, tofs, (const __half*)pgshift(c), pgcur(c), (volatile int*)c->err);
+                   step_seed(c), tclock, tofs, (const __half*)pgshift(c), pgcur(c), err_of(c));
         });
     } else
 #define PFL_ZM(...)                                                                                      \
@@ -628,15 +641,7 @@ bool setup_tma(pfl_ctx* c, int sms) {
   c->encode = (EncodeTiled)fn;
   bool ok = make_maps(c, &c->maps[0], c->ws + c->L.h, c->ws + c->L.g) && make_maps(c, &c->maps[1], c->ws + c->L.h2, c->ws + c->L.g2);
   DISPATCH(c, setup_tma_t, c, sms, &ok);
-  if (!ok || cudaHostAlloc((void**)&c->err, 64, cudaHostAllocPortable) != cudaSuccess) return false;
-  *c->err = 0;
-  return true;
-}
-
-// Releases what the context holds on the host.
-void free_ctx(pfl_ctx* c) {
-  if (c->err) cudaFreeHost(c->err);
-  delete c;
+  return ok && clear_copies(c) == PFL_OK;
 }
 
 // Copy n doubles from a host or device source into the device at dst.
@@ -817,7 +822,6 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
   c->capturing = false;
   c->cap_t0 = 0;
   c->clock_t = -1;
-  c->err = nullptr;
   {
     int sms = 152, per_sm = 2;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
@@ -834,7 +838,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
     c->wide = c->tma < 0 && wide_tile(p);
     if (c->wide) c->zc = z_chunk(p, WIDE_TX, WIDE_TY, (long long)sms * PFL_ZM_MINB, p->nz);
     if (c->tma >= 0 && !setup_tma(c, sms)) {
-      free_ctx(c);
+      delete c;
       return fail(PFL_ERR_CUDA, "setting up the tensor maps of the fused step");
     }
   }
@@ -853,7 +857,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
   for (int a = 0; a < 3; ++a) c->g32.wall[a] = c->geo.wall[a];
   if (c->idx32 && (!fastdiv_ok((unsigned)p->nx, (unsigned)c->geo.N) ||
                    !fastdiv_ok((unsigned)p->ny, (unsigned)(c->geo.N / p->nx)))) {
-    free_ctx(c);
+    delete c;
     return fail(PFL_ERR_STATE, "integer divider self-check failed");
   }
   c->ph.rho_h = p->rho_h;
@@ -878,7 +882,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
       phi_host.resize((size_t)N);
       cudaError_t e = cudaMemcpy(phi_host.data(), phi0, (size_t)N * sizeof(double), cudaMemcpyDeviceToHost);
       if (e != cudaSuccess) {
-        free_ctx(c);
+        delete c;
         return cuda_fail(e, "phi0 to the host for the hydrostatic start");
       }
       ph0 = phi_host.data();
@@ -903,19 +907,19 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
       double* a_p = st + 4 * cnt;
       pfl_status s;
       if ((s = to_device(c, a_phi, phi0 + c0, cnt)) != PFL_OK) {
-        free_ctx(c);
+        delete c;
         return s;
       }
       if (u0 && pass == 1) {
         if ((s = to_device(c, a_ux, u0 + c0, cnt)) != PFL_OK || (s = to_device(c, a_uy, u0 + N + c0, cnt)) != PFL_OK ||
             (s = to_device(c, a_uz, u0 + 2 * N + c0, cnt)) != PFL_OK) {
-          free_ctx(c);
+          delete c;
           return s;
         }
       }
       if (p0) {
         if ((s = to_device(c, a_p, p0 + c0, cnt)) != PFL_OK) {
-          free_ctx(c);
+          delete c;
           return s;
         }
       }
@@ -929,7 +933,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
       cudaError_t e = cudaStreamSynchronize(c->stream);
       if (e == cudaSuccess) e = cudaGetLastError();
       if (e != cudaSuccess) {
-        free_ctx(c);
+        delete c;
         return cuda_fail(e, "initialisation");
       }
     }
@@ -937,7 +941,7 @@ pfl_status pfl_init(const pfl_params* p, const double* phi0, const double* u0, c
   DISPATCH_S(s, c, fresh_phi, c, false);
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (s != PFL_OK || e != cudaSuccess) {
-    free_ctx(c);
+    delete c;
     return s != PFL_OK ? s : cuda_fail(e, "initial phi");
   }
   *out = c;
@@ -950,7 +954,6 @@ pfl_status pfl_step(pfl_ctx* c, int n) {
   CUDA_TRY(on_device.enter(c->device));
   if (n < 0) return fail(PFL_ERR_ARG, "n_steps must be >= 0");
   if (n == 0) return PFL_OK;
-  if (pfl_status e = check_err(c)) return e;
   if (c->zm && c->graph_k > 0 && n >= c->graph_k) {
     // whole graphs of graph_k steps, unless the caller is capturing the stream
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -1007,7 +1010,7 @@ pfl_status pfl_fields(pfl_ctx* c, double* phi, double* rho, double* p, double* u
   }
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return check_err(c);
+  return check_copies(c);
 }
 
 pfl_status pfl_populations(pfl_ctx* c, double* h, double* g) {
@@ -1032,7 +1035,7 @@ pfl_status pfl_populations(pfl_ctx* c, double* h, double* g) {
     }
   }
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return check_err(c);
+  return check_copies(c);
 }
 
 pfl_status pfl_set_populations(pfl_ctx* c, const double* h, const double* g) {
@@ -1053,7 +1056,8 @@ pfl_status pfl_set_populations(pfl_ctx* c, const double* h, const double* g) {
       CUDA_TRY(cudaStreamSynchronize(c->stream));
     }
   }
-  pfl_status s = PFL_OK;
+  pfl_status s = clear_copies(c);
+  if (s != PFL_OK) return s;
   DISPATCH_S(s, c, fresh_phi, c, true);
   if (s != PFL_OK) return s;
   CUDA_TRY(cudaStreamSynchronize(c->stream));
@@ -1141,7 +1145,7 @@ pfl_status pfl_save(pfl_ctx* c, void* buf, size_t bytes) {
     off += hd.bytes[k];
   }
   CUDA_TRY(cudaStreamSynchronize(c->stream));  // the header lives on this stack
-  return check_err(c);
+  return check_copies(c);
 }
 
 pfl_status pfl_load(pfl_ctx* c, const void* buf, size_t bytes) {
@@ -1173,6 +1177,7 @@ pfl_status pfl_load(pfl_ctx* c, const void* buf, size_t bytes) {
   }
   if (bytes < total) return fail(PFL_ERR_ARG, "buffer is shorter than the saved state");
   CUDA_TRY(cudaStreamSynchronize(c->stream));
+  if (pfl_status e = clear_copies(c)) return e;
   // the saved phi buffers keep their roles: buffer `cur` holds phi^t
   const char* from = (const char*)buf + sizeof hd;
   size_t so[NSAVED];
@@ -1237,11 +1242,12 @@ pfl_status pfl_diag(pfl_ctx* c, double out[8], long long* nonfinite) {
     for (int k = 0; k < 8; ++k) out[k] = host[k];
   long long nf = (long long)host[8];
   if (nonfinite) *nonfinite = nf;
+  if (pfl_status e = check_copies(c)) return e;
   if (nf > 0) return fail(PFL_ERR_UNSTABLE, std::to_string(nf) + " cells hold a non-finite phi");
   if (!(umax <= PFL_SPEED_LIMIT))
     return fail(PFL_ERR_UNSTABLE, "flow speed |u| = " + std::to_string(umax) + " exceeds " +
                                       std::to_string(PFL_SPEED_LIMIT) + " (lattice units)");
-  return check_err(c);
+  return PFL_OK;
 }
 
 pfl_status pfl_max_speed(pfl_ctx* c, double* umax) {
@@ -1254,7 +1260,7 @@ pfl_status pfl_max_speed(pfl_ctx* c, double* umax) {
   if (st != PFL_OK) return st;
   CUDA_TRY(cudaMemcpyAsync(umax, ures, sizeof(double), cudaMemcpyDefault, c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return check_err(c);
+  return check_copies(c);
 }
 
 pfl_status pfl_interface_height(pfl_ctx* c, int x, int z, double* y) {
@@ -1269,7 +1275,7 @@ pfl_status pfl_interface_height(pfl_ctx* c, int x, int z, double* y) {
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaMemcpyAsync(y, res, sizeof(double), cudaMemcpyDefault, c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  return check_err(c);
+  return check_copies(c);
 }
 
 pfl_status pfl_kernel_times(pfl_ctx* c, int n, double ms[2]) {
@@ -1455,7 +1461,7 @@ pfl_status zm_step_slots(pfl_ctx* c, const SlotPtr<PREC>& a, const SlotPtr<PREC>
       tma_shape<PREC, QH>(c->tma, [&](auto k) {
         k.launch(c, cfg, m, c->g32, ph, (const typename Store<PREC>::S*)a.h, (const typename Store<PREC>::S*)a.g, b.h, b.g,
                  (const typename Store<PREC>::PhiT*)nullptr, a.phi, c->zc, 0u, (const unsigned long long*)nullptr, 0,
-                 (const __half*)nullptr, (__half*)nullptr, (volatile int*)c->err);
+                 (const __half*)nullptr, (__half*)nullptr, err_of(c));
       });
     }
     return PFL_OK;
@@ -1556,7 +1562,7 @@ pfl_status run_adjoint_zm(pfl_ctx* c, int n, const ObsAt& obs_at, char* aws, con
   if (J) *J = hres[0];
   if (grad)
     for (int k = 0; k < 3; ++k) grad[k] = hres[1 + k];
-  return check_err(c);
+  return check_copies(c);
 }
 
 // The weight field of the observation at step k (relative to the adjoint's
@@ -1728,7 +1734,7 @@ void pfl_destroy(pfl_ctx* c) {
   cudaStreamSynchronize(c->stream);
   drop_graphs(c);
   if (c->cap) cudaStreamDestroy(c->cap);
-  free_ctx(c);
+  delete c;
 }
 
 }  // extern "C"

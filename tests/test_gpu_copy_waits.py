@@ -1,14 +1,20 @@
-"""The waits of the tensor-copy step: a copy that does not arrive ends a wait at its limit, and the
-block waits once more for the same copy before it leaves.
+"""The waits of the tensor-copy step: a copy that does not arrive ends a wait at its limit, the
+block waits once more for the same copy before it leaves, and the library reports the state as
+lost until it is replaced.
 
 The waits (csrc/tma.cuh) run in a kernel of their own, whose copy is withheld, or issued only
-after the first wait has run out; no copy is in flight when a block that gave up ends.
+after the first wait has run out; no copy is in flight when a block that gave up ends.  In the library
+the report word is set from the host.
 """
 import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
+
+from paper_2206_11637_gb300 import _lib as L
+from paper_2206_11637_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
@@ -79,3 +85,29 @@ def test_a_copy_that_does_not_arrive_is_waited_for_twice(waits, late):
     else:
         assert drained == 0 and 20 * MS <= drain_ns + MS < 1000 * MS
     assert none == 1 and none_ns < 20 * MS
+
+
+def test_a_lost_copy_is_reported_until_the_state_is_replaced():
+    from paper_2206_11637_gb300.pflbm import Simulation
+    p = W.Params(128, 96, 44, (1,) * 6, nu_l=0.05)  # tensor copies
+    phi0, u0 = W.sphere(p, (60, 48, 22), 15), W.noise((3,) + p.shape, 5, 1e-2)
+    s, ref = (Simulation(p, phi0, u0, precision="fp32") for _ in range(2))
+    s.step(2)
+    ref.step(2)
+    h, g = s.populations()
+    saved = s.save()
+    for replace in (lambda: s.set_populations(h, g), lambda: s.load(saved)):
+        s.workspace[-128:].view(dtype=s.torch.int32)[0] = 1  # the report word, in the last 256 bytes
+        for call in (lambda: s.step(3), lambda: s.step(40)):  # launches, and a graph replay
+            call()
+            for read in (s.fields, s.populations, s.save, s.max_speed, s.diag, lambda: s.interface_height(0, 0)):
+                with pytest.raises(L.PFLError) as e:
+                    read()
+                assert e.value.status == L.PFL_ERR_CUDA and "did not arrive" in str(e.value)
+        replace()
+        s.fields()
+    assert s.time == ref.time == 2
+    s.step(40)
+    ref.step(40)
+    for a, b in zip(s.populations() + s.fields(), ref.populations() + ref.fields()):
+        assert np.array_equal(a, b)
