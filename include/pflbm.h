@@ -122,6 +122,12 @@ typedef enum { PFL_ENGINE_AUTO = 0, PFL_ENGINE_INPLACE = 1 } pfl_engine;
 /* Device bytes the workspace must hold for these parameters (0 if invalid). */
 size_t pfl_workspace_bytes(const pfl_params* p);
 
+/* The tile that the fused step takes for these parameters, decided on the host:
+ * tile[0] x tile[1] columns per block; tile[2] = 1 where their populations are
+ * read by tensor copies.  Zeros for the in-place engine.  PFL_ERR_ARG for
+ * invalid parameters. */
+pfl_status pfl_step_tile(const pfl_params* p, int tile[3]);
+
 /* The hydrostatic start of pfl_init, on the host: the normalised pressure
  * p* = p / (rho(phi0) c_s^2) of the fluid at rest under gravity, from which
  * the paper starts its gravity cases (sections "Gravity wave", "Rising

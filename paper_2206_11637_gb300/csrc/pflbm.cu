@@ -231,6 +231,9 @@ void launch_phi(pfl_ctx* c) {
   c->cur = 1 - c->cur;
 }
 
+// A launch grid holds at most this many blocks in y and in z (in x 2^31 - 1).
+constexpr long long GRID_YZ = 65535;
+
 // z planes per block of the fused step in tiles of tx x ty, at most `most`.
 // Every block marches zc planes and fills two more (the planes below and above
 // its first) before it starts, about half a plane's work; blocks run in waves
@@ -240,7 +243,7 @@ int z_chunk(const pfl_params* p, int tx, int ty, long long slots, int most) {
   const long long bxy = (long long)((p->nx + tx - 1) / tx) * ((p->ny + ty - 1) / ty);
   int best = std::min(p->nz, most);
   double best_cost = 1e300;
-  for (int zc = best; zc >= 1; --zc) {
+  for (int zc = best; zc >= 1 && (p->nz + zc - 1) / zc <= GRID_YZ; --zc) {
     const long long blocks = bxy * ((p->nz + zc - 1) / zc);
     const double cost = (double)((blocks + slots - 1) / slots) * (zc + 0.5);
     if (cost < best_cost * (1 - 1e-9)) {
@@ -266,7 +269,7 @@ int z_chunk_small(const pfl_params* p, int tx, int ty, long long sms, int reside
   const long long bxy = (long long)((p->nx + tx - 1) / tx) * ((p->ny + ty - 1) / ty);
   int best = p->nz;
   double best_cost = 1e300;
-  for (int zc = best; zc >= 1; --zc) {
+  for (int zc = best; zc >= 1 && (p->nz + zc - 1) / zc <= GRID_YZ; --zc) {
     const long long per_sm = (bxy * ((p->nz + zc - 1) / zc) + sms - 1) / sms;
     const long long rest = per_sm % resident;
     const double cost = (per_sm + (rest == 0 ? 0.0 : rest == 1 ? 0.4 : 0.2)) * (zc + 0.4);
@@ -276,6 +279,13 @@ int z_chunk_small(const pfl_params* p, int tx, int ty, long long sms, int reside
     }
   }
   return best;
+}
+
+// whether tiles of height ty in chunks of at least zc planes fit a launch grid (a
+// tile of 128 x 2 would take more than its blocks in y beyond 131070 rows, where
+// 32 x 8 still fits)
+bool grid_fits(const pfl_params* p, int ty, int zc) {
+  return ((long long)p->ny + ty - 1) / ty <= GRID_YZ && ((long long)p->nz + zc - 1) / zc <= GRID_YZ;
 }
 
 // share of the threads of tx x ty tiles that hold a cell
@@ -292,7 +302,7 @@ double tile_use(const pfl_params* p, int tx, int ty) {
 // gain at the size of L2, bubble 61x183x61 11.7 and 11.8.
 constexpr int WIDE_TX = 64, WIDE_TY = 4;
 bool wide_tile(const pfl_params* p) {
-  return uses_two_arrays(p) && p->precision == PFL_FP32 && p->nz > 1 && qh_of(p) != 9 &&
+  return uses_two_arrays(p) && p->precision == PFL_FP32 && p->nz > 1 && qh_of(p) != 9 && grid_fits(p, WIDE_TY, p->nz) &&
          (long long)p->nx * p->ny * p->nz >= 900000 && tile_use(p, WIDE_TX, WIDE_TY) >= 0.95 * tile_use(p, ZM_TX, ZM_TY);
 }
 
@@ -354,6 +364,7 @@ int tma_tile(const pfl_params* p) {
   int best = -1;
   double most = 0.85 * tile_use(p, ZM_TX, ZM_TY);
   for (int j = 0; j < NTMA; ++j) {
+    if (!grid_fits(p, TMA_TILES[j][1], TMA_ZC)) continue;
     const double r = rate[j] * tile_use(p, TMA_TILES[j][0], TMA_TILES[j][1]);
     if (r > most) {
       most = r;
@@ -768,6 +779,18 @@ const char* pfl_last_error(void) { return g_err.c_str(); }
 size_t pfl_workspace_bytes(const pfl_params* p) {
   if (!check_params(p).empty()) return 0;
   return layout_of(p).total;
+}
+
+pfl_status pfl_step_tile(const pfl_params* p, int tile[3]) {
+  if (!p || !tile) return fail(PFL_ERR_ARG, "params and tile must not be NULL");
+  const std::string why = check_params(p);
+  if (!why.empty()) return fail(PFL_ERR_ARG, why);
+  const int j = tma_tile(p);
+  const bool fused = uses_two_arrays(p), wide = wide_tile(p);
+  tile[0] = j >= 0 ? TMA_TILES[j][0] : wide ? WIDE_TX : fused ? ZM_TX : 0;
+  tile[1] = j >= 0 ? TMA_TILES[j][1] : wide ? WIDE_TY : fused ? zm_ty(p->nz == 1) : 0;
+  tile[2] = j >= 0;
+  return PFL_OK;
 }
 
 pfl_status pfl_hydrostatic_pstar(const pfl_params* p, const double* phi0, double* pstar) {

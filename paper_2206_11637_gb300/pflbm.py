@@ -45,6 +45,15 @@ def workspace_bytes(p, precision):
     return L.load().pfl_workspace_bytes(ctypes.byref(s))
 
 
+def step_tile(p, precision):
+    """(width, height, tensor copies) of the fused step's tile for these
+    parameters (pfl_step_tile, on the host); zeros for the in-place engine."""
+    s = _params_struct(p, precision)
+    tile = np.zeros(3, dtype=np.intc)
+    L.check(L.load().pfl_step_tile(ctypes.byref(s), _ptr(tile)))
+    return int(tile[0]), int(tile[1]), bool(tile[2])
+
+
 def hydrostatic_pstar(p, phi0):
     """The library's hydrostatic start (pfl_hydrostatic_pstar, on the host):
     p* of the fluid at rest under p.gravity, zero pressure at p.p_level along
