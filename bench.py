@@ -112,9 +112,14 @@ def workload(name):
     raise SystemExit("unknown workload " + name)
 
 
+# what the step's launches are made of: its kernels, and the host code that picks
+# their tiles and z chunks
+KERNEL_SOURCES = ("kernels.cuh", "lattice.cuh", "step.cuh", "moments.cuh", "vec.cuh", "tma.cuh", "pflbm.cu")
+
+
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("kernels.cuh", "lattice.cuh", "step.cuh"):
+    for f in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_2206_11637_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
