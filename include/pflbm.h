@@ -250,8 +250,9 @@ pfl_status pfl_kernel_times(pfl_ctx* ctx, int n_steps, double ms[2]);
 
 /* Device bytes of the adjoint workspace for an adjoint over n_steps steps
  * (0 if ctx is NULL or n_steps < 1).  It holds ceil(n_steps / K) checkpoints
- * and K recomputed states with K = ceil(sqrt(n_steps)), two adjoint
- * population sets, the observation weights and the reduction scratch. */
+ * and K - 1 recomputed states (in-place engine: K, and the final state) with
+ * K = ceil(sqrt(n_steps)), two adjoint population sets, the observation weights
+ * and the reduction scratch. */
 size_t pfl_adjoint_workspace_bytes(const pfl_ctx* ctx, int n_steps);
 
 /* Discrete adjoint of n_steps time steps from the current state: the gradient

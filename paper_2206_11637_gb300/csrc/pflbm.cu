@@ -1368,7 +1368,8 @@ AdjLayout adj_layout(const pfl_ctx* c, int n) {
   A.ck = off;
   off += (size_t)A.nck * A.state;
   A.seg = off;
-  off += (size_t)A.K * A.state;
+  // (the fused engine's segments start in their checkpoint)
+  off += (size_t)(c->zm ? A.K - 1 : A.K) * A.state;
   A.fin = off;
   if (!c->zm) off += A.state;  // the fused engine's reverse sweep leaves the live state alone
   A.lam0 = off;
@@ -1563,7 +1564,7 @@ pfl_status run_adjoint_zm(pfl_ctx* c, int n, const ObsAt& obs_at, char* aws, con
     const int k0 = sgm * A.K, k1 = (k0 + A.K < n) ? k0 + A.K : n;
     // state k of the segment: its first in the checkpoint, the others in their slots
     auto slot = [&](int k) {
-      return aws + (k == k0 ? A.ck + (size_t)sgm * A.state : A.seg + (size_t)(k - k0) * A.state);
+      return aws + (k == k0 ? A.ck + (size_t)sgm * A.state : A.seg + (size_t)(k - k0 - 1) * A.state);
     };
     for (int k = k0; k + 1 < k1; ++k) {
       const pfl_status s = zm_step_slots<PREC, QH>(c, SlotPtr<PREC>(c, slot(k)), SlotPtr<PREC>(c, slot(k + 1)));
