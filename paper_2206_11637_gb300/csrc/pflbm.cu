@@ -431,8 +431,7 @@ void step_only(pfl_ctx* c) {
     if (c->tma >= 0) {
       if constexpr (has_tma<PREC, QH>())
         tma_shape<PREC, QH>(c->tma, [&](auto k) {
-          k.launch(c, cfg, c->maps[c->ab], c->g32, ph1, ha, ga, hnext<PREC>(c), gnext<PREC>(c), shift, phicur<PREC>(c), c->zc,
-                   step_seed(c), tclock, tofs, (const __half*)pgshift(c), pgcur(c), err_of(c));
+          k.launch(c, cfg, c->maps[c->ab], c->g32, ph1, ha, ga, hnext<PREC>(c), gnext<PREC>(c), phicur<PREC>(c), c->zc, err_of(c));
         });
     } else
 #define PFL_ZM(...)                                                                                      \
@@ -1484,8 +1483,7 @@ pfl_status zm_step_slots(pfl_ctx* c, const SlotPtr<PREC>& a, const SlotPtr<PREC>
       cfg.stream = c->stream;
       tma_shape<PREC, QH>(c->tma, [&](auto k) {
         k.launch(c, cfg, m, c->g32, ph, (const typename Store<PREC>::S*)a.h, (const typename Store<PREC>::S*)a.g, b.h, b.g,
-                 (const typename Store<PREC>::PhiT*)nullptr, a.phi, c->zc, 0u, (const unsigned long long*)nullptr, 0,
-                 (const __half*)nullptr, (__half*)nullptr, err_of(c));
+                 a.phi, c->zc, err_of(c));
       });
     }
     return PFL_OK;

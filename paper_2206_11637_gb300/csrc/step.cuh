@@ -1325,9 +1325,8 @@ __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
     k_step_tma(const __grid_constant__ StepMaps maps, Geo32 geo, typename StepV<PREC>::Par ph,
                const typename Store<PREC>::S* __restrict__ hA, const typename Store<PREC>::S* __restrict__ gA,
                typename Store<PREC>::S* __restrict__ hB, typename Store<PREC>::S* __restrict__ gB,
-               const typename Store<PREC>::PhiT* __restrict__ phi_shift,
-               typename Store<PREC>::PhiT* __restrict__ phi_out, int zc, unsigned seed, const unsigned long long* tclock,
-               int tofs, const __half* __restrict__ pg_in, __half* __restrict__ pg_out, volatile int* err) {
+               typename Store<PREC>::PhiT* __restrict__ phi_out, int zc, volatile int* err) {
+  static_assert(PREC != 2, "FP16S is bound by instruction issue and takes no copies");
   __shared__ unsigned long long mbar[2];
   const unsigned bar = smem_u32(mbar);
   if (threadIdx.x == 0 && threadIdx.y == 0) {
@@ -1337,8 +1336,7 @@ __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
   const int lost = __syncthreads_or(*err);
   if (PFL_ZM_PDL) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (lost) return;
-  if (PREC == 2 && tclock) seed = step_seed_of(*tclock + (unsigned long long)tofs);
-  if (!zm_tile<PREC, QH, TY, 0, 0, TX, 1>(geo, ph, hA, gA, hB, gB, phi_shift, phi_out, zc, seed, nullptr, pg_in, pg_out,
+  if (!zm_tile<PREC, QH, TY, 0, 0, TX, 1>(geo, ph, hA, gA, hB, gB, nullptr, phi_out, zc, 0u, nullptr, nullptr, nullptr,
                                           blockIdx.x, blockIdx.y, blockIdx.z, &maps, bar) &&
       threadIdx.x == 0 && threadIdx.y == 0)
     *err = 1;
