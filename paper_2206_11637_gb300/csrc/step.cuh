@@ -44,11 +44,13 @@
 #define PFL_ZM_MINB_FP64 2
 #endif
 // L1 prefetch of the g populations of the plane the fused FP32 step collides
-// next, issued one plane ahead right after the plane barrier (1; 0 = none).
-// Measured on the 128x384x128 bubble: FP32 14.0 -> 14.9 GLUPS.  FP16S (issue
-// bound) lost 5 %, single-plane lattices 8-10 % and the D3Q27 phase field 1 %
-// (10.94 -> 10.82), so they take none.  (The h populations of the plane filled
-// next as well: 15.0 -> 12.5 GLUPS on a 256x192x256 impact.)
+// next, issued one plane ahead right after the plane barrier (1; 0 = none), in
+// tiles without tensor copies.  us per step with and without: drop 96^3 (32 x 8)
+// 59.7 and 61.7, bubble 96x250x99 169.3 and 177.4; bubble 61x183x61 and the Taylor
+// tubes equal within 0.5 %; drop 32^3, in L2 anyway, 5.71 and 5.01.  FP16S (issue
+// bound) lost 5 %, single-plane lattices 8-10 % and the D3Q27 phase field 1 %, so
+// they take none.  (The h populations of the plane filled next as well: 15.0 ->
+// 12.5 GLUPS on a 256x192x256 impact.)
 #ifndef PFL_ZM_PREFETCH
 #define PFL_ZM_PREFETCH 1
 #endif
@@ -1097,18 +1099,18 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
   extern __shared__ __align__(128) unsigned char dyn[];
   S* sG = (S*)dyn;
   S* sH = sG + QG * NT;
-  CopyGate gate_h{mbar}, gate_g{mbar + 8};
+  const unsigned mbar_h = mbar, mbar_g = mbar + 8;
   bool ok = true;
   auto issue_h = [&](int zp) {
     if (tid == 0) {
-      mbar_expect(gate_h.bar, QH * NT * sizeof(S));
-      tma4(smem_u32(sH), &maps->h, x0, y0, wrap_or_clamp(zp, (int)geo.nz, geo.wall[2]), 0, gate_h.bar);
+      mbar_expect(mbar_h, QH * NT * sizeof(S));
+      tma4(smem_u32(sH), &maps->h, x0, y0, wrap_or_clamp(zp, (int)geo.nz, geo.wall[2]), 0, mbar_h);
     }
   };
   auto issue_g = [&](int z) {
     if (tid == 0) {
-      mbar_expect(gate_g.bar, QG * NT * sizeof(S));
-      tma4(smem_u32(sG), &maps->g, x0, y0, z, 0, gate_g.bar);
+      mbar_expect(mbar_g, QG * NT * sizeof(S));
+      tma4(smem_u32(sG), &maps->g, x0, y0, z, 0, mbar_g);
     }
   };
 
@@ -1133,20 +1135,24 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
   // FP16S finds its ring cell once (bubble 128x384x128: 410 -> 398 us per step; FP64
   // is indifferent, and FP32 planes lose, 5.65 -> 5.84 us on 200x400).
   static_assert(!F16 || NRING <= NT, "one ring cell per thread");
-  const RingCell own_ring = ring_cell(min(tid, NRING - 1));
+  const RingCell own_ring = F16 ? ring_cell(min(tid, NRING - 1)) : RingCell{};
   // phi of plane zp over the tile (with the h moments of the own cells) and its ring
   auto fill = [&](int zp, int slot, int pslot, int mslot) {
     const unsigned zq = (unsigned)wrap_or_clamp(zp, (int)geo.nz, geo.wall[2]);
     const unsigned c = xq + geo.nx * (yq + geo.ny * zq);
     CellOff o;
     if (F16) o = off_xyz(geo, xq, yq, zq, SOLID ? __ldg(links + c) : 0u);
-    RingCell rc = {};
+    // phi of ring cell r and its place
+    auto ring_phi = [&](int r, int& at, PhiT& v) {
+      const RingCell q = F16 ? own_ring : ring_cell(r);
+      at = q.at;
+      v = phi_at(q.x, q.y, zq);
+      if constexpr (F16) pring[pslot][at] = ld_pshift(pg_in, q.x + geo.nx * (q.y + geo.ny * zq));
+    };
+    int rat = 0;
     PhiT rv = 0;
-    if constexpr (RING1ST) {
-      rc = ring_cell(min(tid, NRING - 1));
-      rv = phi_at(rc.x, rc.y, zq);
-    }
-    if constexpr (TM != 0) ok = gate_h.wait() && ok;
+    if constexpr (RING1ST) ring_phi(NRING < NT ? min(tid, NRING - 1) : tid, rat, rv);
+    if constexpr (TM != 0) ok = copy_wait(mbar_h, zp - (z0 - 1)) && ok;
     if (PREC == 0 && !FLAT && (zp < z0 || zp >= z1)) {
       // FP64, the planes beside the chunk: their cells collide in other blocks, so
       // phi alone (14 additions instead of 39): drop 32^3, one plane per chunk,
@@ -1177,13 +1183,12 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
       hm[9 * NT] = m.xz;
     }
     if constexpr (F16) pring[pslot][i0] = ld_pshift(pg_in, c);
-    if (RING1ST && tid < NRING) ring[slot][rc.at] = rv;
+    if (RING1ST && tid < NRING) ring[slot][rat] = rv;
 #pragma unroll
     for (int r0 = RING1ST ? NT : 0; r0 < NRING; r0 += NT) {
       if (r0 + tid < NRING) {
-        const RingCell q = F16 ? own_ring : ring_cell(r0 + tid);
-        ring[slot][q.at] = phi_at(q.x, q.y, zq);
-        if constexpr (F16) pring[pslot][q.at] = ld_pshift(pg_in, q.x + geo.nx * (q.y + geo.ny * zq));
+        ring_phi(r0 + tid, rat, rv);
+        ring[slot][rat] = rv;
       }
     }
   };
@@ -1227,14 +1232,13 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
     const int z = FLAT ? zp : zp - 1;
     const int bp = zp - (z0 - 1), b = bp - 1;  // plane counts from z0 - 1
     cell = (unsigned)x + geo.nx * ((unsigned)y + geo.ny * (unsigned)z);
-    if (TM && z >= z0) ok = gate_g.wait() && ok;
+    if (TM) ok = copy_wait(mbar_g, z - z0) && ok;
     if (EARLY && z >= z0 && (TM || active)) gather_g(b);
     fill(FLAT ? 0 : zp, FLAT ? 0 : bp % NS, FLAT ? 0 : bp % NSP, FLAT ? 0 : bp & 1);
     if constexpr (TM != 0) {
       if (!__syncthreads_and(ok)) {
-        // (every copy issued so far has been waited for)
-        gate_h.drain();
-        gate_g.drain();
+        copy_wait(mbar_h, bp);  // (no other copy has been issued)
+        copy_wait(mbar_g, z - z0);
         return false;
       }
       if (zp < z1) issue_h(zp + 1);
@@ -1319,7 +1323,7 @@ __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
 // when a copy did not arrive; the state is lost then, and blocks that find it set
 // return at once, so that later waves, steps and graph replays do not each wait for
 // their copies' limit.  (Read before the wait for the previous step, whose time
-// hides it: bubble 128x384x128 363.6 us per step without, 364.2 with.)
+// hides it: bubble 128x384x128 365.3 us per step without, 365.5 with.)
 template <int PREC, int QH, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
     k_step_tma(const __grid_constant__ StepMaps maps, Geo32 geo, typename StepV<PREC>::Par ph,

@@ -21,41 +21,41 @@ pytestmark = pytest.mark.gpu
 KERNEL = r"""
 #include "tma.cuh"
 using namespace pfl;
-// res: first wait, its ns, drain, its ns, drain of a barrier without copies, its ns
-__global__ void k_waits(const int* src, int late, unsigned long long limit, unsigned long long* res) {
+// res: first wait, its ns, second wait, its ns, wait at a barrier without copies, its ns, the value copied
+__global__ void k_waits(const int* src, int late, unsigned limit, unsigned* res) {
   __shared__ unsigned long long mbar[2];
   __shared__ __align__(16) int dst[4];
-  CopyGate a{smem_u32(mbar)}, b{smem_u32(mbar + 1)};
+  const unsigned a = smem_u32(mbar), b = smem_u32(mbar + 1);
   if (threadIdx.x == 0) {
-    mbar_init(a.bar);
-    mbar_init(b.bar);
-    mbar_expect(a.bar, 16);
+    mbar_init(a);
+    mbar_init(b);
+    mbar_expect(a, 16);
   }
   __syncthreads();
-  const unsigned long long t0 = timer_ns();
-  const bool w = a.wait(limit);
-  const unsigned long long t1 = timer_ns();
+  const unsigned t0 = timer_ns();
+  const bool w = copy_wait(a, 0, limit);
+  const unsigned t1 = timer_ns();
   __syncthreads();
   if (late && threadIdx.x == 0)
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], 16, [%2];" ::"r"(smem_u32(dst)),
-                 "l"(src), "r"(a.bar) : "memory");
-  const unsigned long long t2 = timer_ns();
-  const bool d = a.drain(limit);
-  const unsigned long long t3 = timer_ns();
-  const bool e = b.drain(limit);
-  const unsigned long long t4 = timer_ns();
+                 "l"(src), "r"(a) : "memory");
+  const unsigned t2 = timer_ns();
+  const bool d = copy_wait(a, 0, limit);
+  const unsigned t3 = timer_ns();
+  const bool e = copy_wait(b, -1, limit);
+  const unsigned t4 = timer_ns();
   if (threadIdx.x == 0) {
-    const unsigned long long v[7] = {w, t1 - t0, d, t3 - t2, e, t4 - t3, d ? (unsigned long long)dst[0] : 0};
+    const unsigned v[7] = {w, t1 - t0, d, t3 - t2, e, t4 - t3, d ? (unsigned)dst[0] : 0};
     for (int k = 0; k < 7; ++k) res[k] = v[k];
   }
 }
-extern "C" int run_waits(int late, unsigned long long limit, unsigned long long* out) {
+extern "C" int run_waits(int late, unsigned limit, unsigned* out) {
   int *src, one[4] = {41, 0, 0, 0};
-  unsigned long long* res;
-  if (cudaMalloc(&src, 16) != cudaSuccess || cudaMalloc(&res, 56) != cudaSuccess) return 1;
+  unsigned* res;
+  if (cudaMalloc(&src, 16) != cudaSuccess || cudaMalloc(&res, 28) != cudaSuccess) return 1;
   cudaMemcpy(src, one, 16, cudaMemcpyHostToDevice);
   k_waits<<<1, 64>>>(src, late, limit, res);
-  const cudaError_t e = cudaMemcpy(out, res, 56, cudaMemcpyDeviceToHost);
+  const cudaError_t e = cudaMemcpy(out, res, 28, cudaMemcpyDeviceToHost);
   cudaFree(src);
   cudaFree(res);
   return (int)e;
@@ -76,8 +76,8 @@ def waits(tmp_path_factory):
 
 @pytest.mark.parametrize("late", [0, 1])
 def test_a_copy_that_does_not_arrive_is_waited_for_twice(waits, late):
-    out = (ctypes.c_ulonglong * 7)()
-    assert waits.run_waits(late, ctypes.c_ulonglong(20 * MS), out) == 0
+    out = (ctypes.c_uint * 7)()
+    assert waits.run_waits(late, ctypes.c_uint(20 * MS), out) == 0
     arrived, ns, drained, drain_ns, none, none_ns, value = list(out)
     assert arrived == 0 and 20 * MS <= ns + MS < 1000 * MS  # the limit, to the timer's step
     if late:
