@@ -131,13 +131,13 @@ def kernel_hash():
 # kernel version does not apply.
 NCU_TRAFFIC = {
     # k_step_zm<2, 15, 0, 0> (FP16S) captured on the half-size impact (256x192x256,
-    # 12.58 M cells): 1.1690 GB read + 1.0996 GB written = 180.3 B/cell; the
+    # 12.58 M cells): 1.1684 GB read + 1.0946 GB written = 179.9 B/cell; the
     # launch's traffic grows with the cells it updates, so a full 100.7 M-cell
-    # launch moves 180.3 x 100.66 M = 18.15 GB
+    # launch moves 179.9 x 100.66 M = 18.10 GB
     # (profiles/k_step_tma_zm_drop_impact_256x192x256.md)
-    ("drop_impact", "fp16s", "084656e12a3aaa0d"): 1.8149e10,
-    # k_step_tma<1, 15, 128, 2> (FP32) on the same case: 2.2430 + 2.1202 GB = 346.7 B/cell
-    ("drop_impact", "fp32", "084656e12a3aaa0d"): 3.4905e10,
+    ("drop_impact", "fp16s", "c29c4b46e4549ee6"): 1.8104e10,
+    # k_step_tma<1, 15, 128, 2> (FP32) on the same case: 2.2434 + 2.1202 GB = 346.8 B/cell
+    ("drop_impact", "fp32", "c29c4b46e4549ee6"): 3.4909e10,
 }
 
 # Warp instructions per launch of the same kernels (smsp__inst_executed.sum of
@@ -145,8 +145,8 @@ NCU_TRAFFIC = {
 # side of the roofline: launches that issue more than they move (FP16S) are
 # bound there.
 NCU_INST = {
-    ("drop_impact", "fp16s", "084656e12a3aaa0d"): 5.2956e9,    # 52.61 per cell
-    ("drop_impact", "fp32", "084656e12a3aaa0d"): 4.5269e9,     # 44.97 per cell
+    ("drop_impact", "fp16s", "c29c4b46e4549ee6"): 5.2621e9,    # 52.27 per cell
+    ("drop_impact", "fp32", "c29c4b46e4549ee6"): 4.4225e9,     # 43.93 per cell
 }
 
 

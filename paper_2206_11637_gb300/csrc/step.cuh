@@ -1157,8 +1157,9 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
       // FP64, the planes beside the chunk: their cells collide in other blocks, so
       // phi alone (14 additions instead of 39): drop 32^3, one plane per chunk,
       // 47.7 -> 43.9 us per step, 64^3 295 -> 288, bubble 61x183x61 742 -> 728, D3Q27
-      // drop 48^3 190 -> 178.  FP32 and FP16S do not wait for the additions and
-      // lose 3 % by the second code site.
+      // drop 48^3 190 -> 178 (with moments by axes; 44.9, 753 and 187 with those by
+      // pairs).  FP32 and FP16S do not wait for the additions and lose 3 % by the second
+      // code site.
       ring[slot][i0] = phi_at(xq, yq, zq);
     } else {
       const Mom<V> m = set_moments<PREC, QH>(
@@ -1323,7 +1324,7 @@ __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
 // when a copy did not arrive; the state is lost then, and blocks that find it set
 // return at once, so that later waves, steps and graph replays do not each wait for
 // their copies' limit.  (Read before the wait for the previous step, whose time
-// hides it: bubble 128x384x128 365.3 us per step without, 365.5 with.)
+// hides it: bubble 128x384x128 365.0 us per step without, 365.6 with.)
 template <int PREC, int QH, int TX, int TY>
 __global__ void __launch_bounds__(TX* TY, zm_minb(PREC, TX* TY))
     k_step_tma(const __grid_constant__ StepMaps maps, Geo32 geo, typename StepV<PREC>::Par ph,
