@@ -114,7 +114,7 @@ def workload(name):
 
 # what the step's launches are made of: its kernels, and the host code that picks
 # their tiles and z chunks
-KERNEL_SOURCES = ("kernels.cuh", "lattice.cuh", "step.cuh", "moments.cuh", "vec.cuh", "tma.cuh", "pflbm.cu")
+KERNEL_SOURCES = ("kernels.cuh", "lattice.cuh", "step.cuh", "vec.cuh", "tma.cuh", "pflbm.cu")
 
 
 def kernel_hash():
@@ -135,9 +135,9 @@ NCU_TRAFFIC = {
     # launch's traffic grows with the cells it updates, so a full 100.7 M-cell
     # launch moves 179.9 x 100.66 M = 18.10 GB
     # (profiles/k_step_tma_zm_drop_impact_256x192x256.md)
-    ("drop_impact", "fp16s", "c29c4b46e4549ee6"): 1.8104e10,
+    ("drop_impact", "fp16s", "ce538975ede1cf2f"): 1.8104e10,
     # k_step_tma<1, 15, 128, 2> (FP32) on the same case: 2.2434 + 2.1202 GB = 346.8 B/cell
-    ("drop_impact", "fp32", "c29c4b46e4549ee6"): 3.4909e10,
+    ("drop_impact", "fp32", "ce538975ede1cf2f"): 3.4909e10,
 }
 
 # Warp instructions per launch of the same kernels (smsp__inst_executed.sum of
@@ -145,8 +145,8 @@ NCU_TRAFFIC = {
 # side of the roofline: launches that issue more than they move (FP16S) are
 # bound there.
 NCU_INST = {
-    ("drop_impact", "fp16s", "c29c4b46e4549ee6"): 5.2621e9,    # 52.27 per cell
-    ("drop_impact", "fp32", "c29c4b46e4549ee6"): 4.4225e9,     # 43.93 per cell
+    ("drop_impact", "fp16s", "ce538975ede1cf2f"): 5.2621e9,    # 52.27 per cell
+    ("drop_impact", "fp32", "ce538975ede1cf2f"): 4.4225e9,     # 43.93 per cell
 }
 
 

@@ -23,7 +23,6 @@
 #pragma once
 
 #include "kernels.cuh"
-#include "moments.cuh"
 #include "tma.cuh"
 #include "vec.cuh"
 
@@ -285,12 +284,112 @@ __device__ __forceinline__ void load_pair(const typename Store<PREC>::S* __restr
 
 
 // ---------------------------------------------------------------------------
-// Moments (of FP64: moments.cuh).
+// Moments (FP64).  A population set is a tensor product (D3Q27, D2Q9) or its axis
+// and corner part (D3Q15), so the moments up to second order fall out of sums and
+// differences along x, then y, then z: 66 operations for the ten moments of
+// D3Q27 against 111 by opposite pairs, 39 against 63 for D3Q15.  The first moments
+// along y and z are differences of sums at the size of p*, so by themselves they
+// round at that size (5e-17 off at p* = 5, |u| = 1e-3) where those along x, and
+// all three by pairs, are exact.  The populations they are made of are rounded
+// at that size already: against 80-bit arithmetic a step's u is nearer than with the
+// moments by pairs one by one (walled pool, x, y, z: 3.7, 6.9, 6.1e-17 and 4.8, 9.4,
+// 7.1e-17; drop 4.8e-19 and 5.0 to 5.2e-19), phi and p are the same to 2 %.  Sums
+// and differences of the pairs first, with shared partial sums (81 operations),
+// gave the same errors within 5 % for 3 to 5 % more time (drop 32^3 43.5 and
+// 44.9 us per step, bubble 61x183x61 728 and 753).
+// ld(cx, cy, cz) gives the population of direction c.
+template <class V>
+struct Mom {
+  V s, x, y, z, xx, yy, zz, xy, yz, xz;  // sum f, sum c f, sum c c f
+};
 // index of direction c in the lattice's order
 template <int Q>
 __host__ __device__ constexpr int lq_index(int cx, int cy, int cz) {
   const int i = 9 * (cz + 1) + 3 * (cy + 1) + cx + 1;
   return Q == 27 ? i : (Q == 9 ? i - 9 : (i < 13 ? i / 2 : (i == 13 ? 7 : i / 2 + 1)));
+}
+
+template <class V>
+__device__ __forceinline__ V sum3(V a, V b, V c) {
+  return (a + c) + b;
+}
+
+template <class V>
+struct PlaneMom {
+  V m00, m10, m20, m01, m11, m02;  // x-order, y-order within one z plane
+};
+template <class V, class LD>
+__device__ __forceinline__ PlaneMom<V> plane_mom(const LD& ld, int cz) {
+  V a0[3], a1[3], a2[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const V l = ld(-1, j - 1, cz), c = ld(0, j - 1, cz), r = ld(1, j - 1, cz);
+    a0[j] = sum3(l, c, r);
+    a1[j] = r - l;
+    a2[j] = l + r;
+  }
+  PlaneMom<V> p;
+  p.m00 = sum3(a0[0], a0[1], a0[2]);
+  p.m01 = a0[2] - a0[0];
+  p.m02 = a0[0] + a0[2];
+  p.m10 = sum3(a1[0], a1[1], a1[2]);
+  p.m11 = a1[2] - a1[0];
+  p.m20 = sum3(a2[0], a2[1], a2[2]);
+  return p;
+}
+
+template <int Q, class V, class LD>
+__device__ __forceinline__ Mom<V> moments(const LD& ld) {
+  Mom<V> m;
+  if constexpr (Q == 27) {
+    const PlaneMom<V> a = plane_mom<V>(ld, -1), b = plane_mom<V>(ld, 0), c = plane_mom<V>(ld, 1);
+    m.s = sum3(a.m00, b.m00, c.m00);
+    m.z = c.m00 - a.m00;
+    m.zz = a.m00 + c.m00;
+    m.x = sum3(a.m10, b.m10, c.m10);
+    m.xz = c.m10 - a.m10;
+    m.y = sum3(a.m01, b.m01, c.m01);
+    m.yz = c.m01 - a.m01;
+    m.xx = sum3(a.m20, b.m20, c.m20);
+    m.yy = sum3(a.m02, b.m02, c.m02);
+    m.xy = sum3(a.m11, b.m11, c.m11);
+  } else if constexpr (Q == 9) {
+    const PlaneMom<V> b = plane_mom<V>(ld, 0);
+    m.s = b.m00;
+    m.x = b.m10;
+    m.y = b.m01;
+    m.xx = b.m20;
+    m.yy = b.m02;
+    m.xy = b.m11;
+    m.z = m.zz = m.yz = m.xz = vbc<V>(0.0);
+  } else {
+    PlaneMom<V> p[2];  // corners of the planes cz = -1, 1: m00, m10, m01, m11
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const V a = ld(-1, -1, 2 * k - 1), b = ld(1, -1, 2 * k - 1), c = ld(-1, 1, 2 * k - 1), d = ld(1, 1, 2 * k - 1);
+      const V r0 = a + b, r1 = c + d, e0 = b - a, e1 = d - c;
+      p[k].m00 = r0 + r1;
+      p[k].m01 = r1 - r0;
+      p[k].m10 = e0 + e1;
+      p[k].m11 = e1 - e0;
+    }
+    const V c0 = p[0].m00 + p[1].m00;
+    const V xm = ld(-1, 0, 0), xp = ld(1, 0, 0), ym = ld(0, -1, 0), yp = ld(0, 1, 0), zm = ld(0, 0, -1),
+            zp = ld(0, 0, 1), r = ld(0, 0, 0);
+    const V sx = xm + xp, sy = ym + yp, sz = zm + zp, dx = xp - xm, dy = yp - ym, dz = zp - zm;
+    const V cx = p[0].m10 + p[1].m10, cy = p[0].m01 + p[1].m01, cz = p[1].m00 - p[0].m00;
+    m.s = (c0 + ((sx + sy) + sz)) + r;
+    m.x = cx + dx;
+    m.y = cy + dy;
+    m.z = cz + dz;
+    m.xx = c0 + sx;
+    m.yy = c0 + sy;
+    m.zz = c0 + sz;
+    m.xy = p[0].m11 + p[1].m11;
+    m.xz = p[1].m10 - p[0].m10;
+    m.yz = p[1].m01 - p[0].m01;
+  }
+  return m;
 }
 
 // FP32 moments by opposite pairs, in the order of the set's members: S = f_c +
@@ -619,8 +718,8 @@ __device__ __forceinline__ void collide(const PhysV<V>& ph, V pc, const Grad<V>&
     const V dzz = QG == 9 ? vbc<V>(0.0) : vfma(vfma(three, gm.zz, mp), third, qz);  // 2-D: the trace runs over x and y
     const V a2 = vfma(vbc<V>(-4.5), omega, vbc<V>(4.5));
     const V al = vfma(vbc<V>(1.5), (qx + qy) + qz, (a2 * vbc<V>(-1.0 / 3.0)) * ((dxx + dyy) + dzz));
-    const V fr = vquot(vbc<V>(1.5), rho, rinv);
-    const V bx = vfma(fr, Fx, three * ux), by = vfma(fr, Fy, three * uy), bz = vfma(fr, Fz, three * uz);
+    const V fr = vbc<V>(1.5) * rinv, k3 = three;
+    const V bx = vfma(fr, Fx, k3 * ux), by = vfma(fr, Fy, k3 * uy), bz = vfma(fr, Fz, k3 * uz);
     const V k45 = vbc<V>(-4.5), k9 = vbc<V>(-9.0), a22 = a2 + a2;
     const V Gxx = vfma(k45, qx, a2 * dxx), Gyy = vfma(k45, qy, a2 * dyy), Gzz = vfma(k45, qz, a2 * dzz);
     const V qxy = mx * uy, qyz = my * uz, qxz = mx * uz;
@@ -1157,9 +1256,8 @@ __device__ __forceinline__ bool zm_tile(const Geo32& geo, const typename StepV<P
       // FP64, the planes beside the chunk: their cells collide in other blocks, so
       // phi alone (14 additions instead of 39): drop 32^3, one plane per chunk,
       // 47.7 -> 43.9 us per step, 64^3 295 -> 288, bubble 61x183x61 742 -> 728, D3Q27
-      // drop 48^3 190 -> 178 (with moments by axes; 44.9, 753 and 187 with those by
-      // pairs).  FP32 and FP16S do not wait for the additions and lose 3 % by the second
-      // code site.
+      // drop 48^3 190 -> 178.  FP32 and FP16S do not wait for the additions and
+      // lose 3 % by the second code site.
       ring[slot][i0] = phi_at(xq, yq, zq);
     } else {
       const Mom<V> m = set_moments<PREC, QH>(

@@ -49,14 +49,4 @@ __device__ __forceinline__ F1 vdiv(F1 a, F1 b) { return F1{__fdiv_rn(a.v, b.v)};
 __device__ __forceinline__ D1 vsqrt(D1 a) { return D1{__dsqrt_rn(a.v)}; }
 __device__ __forceinline__ F1 vsqrt(F1 a) { return F1{__fsqrt_rn(a.v)}; }
 
-// a / b from r = 1 / b rounded to nearest: the product a r, corrected by its
-// residual, which the fused multiply-add forms in one rounding (P. W. Markstein,
-// IBM J. Res. Dev. 34, 1990).  Half an ulp, like the quotient, where a r alone
-// rounds twice.
-template <class V>
-__device__ __forceinline__ V vquot(V a, V b, V r) {
-  const V q = a * r;
-  return vfma(vfma(-b, q, a), r, q);
-}
-
 }  // namespace pfl
